@@ -81,7 +81,156 @@ void dev_free(casimir_ctx *c, void *p)
 // plan preparation (host)
 // ---------------------------------------------------------------------------------
 
-static int prepare_plan(casimir_plan_t *P)
+// Entry tables of a 2D TM/TE plan for the resident march of shape q: the rows each warp of a simulation's
+// cluster stages, and the entries of each CTA, one per thread.  False when the shape cannot hold them
+// (more entries than threads in a CTA, staged rows and coefficients beyond the shared memory left, or sums beyond the second
+// field buffer, where they wait between launches).
+static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
+{
+    const PlanData &D = P->data;
+    const int cx = q->fp64 ? 2 : 4, nwarp = q->threads / 32, nx = D.prob.n[0], ny = D.prob.n[1];
+    const int64_t N = (int64_t)nx * ny;
+    P->resW.clear();
+    P->resC.clear();
+    P->resE.clear();
+    q->stage_words = q->ne_max = 0;
+    if ((int64_t)q->cluster * 16 + 16 > 3 * N * (int64_t)P->rsize) return false;
+    // the cluster's first row: the first that leaves the rows of every horizontal face in one CTA
+    std::map<int, std::pair<int, int>> span;   // face -> its measured rows
+    for (const Sim &sm : D.sims)
+        if (D.faces[sm.face].axis == 1)
+            for (const Entry &e : sm.meas) {
+                const int j = (int)(e.idx / nx);
+                auto it = span.emplace(sm.face, std::make_pair(j, j)).first;
+                it->second.first = std::min(it->second.first, j);
+                it->second.second = std::max(it->second.second, j);
+            }
+    auto cta_of = [&](int row) {
+        const int b = (int)(((int64_t)(row + 1) * q->nb - 1) / ny);   // y0(b) = b ny / nb <= row
+        return (int)(((int64_t)(b + 1) * q->cluster - 1) / q->nb);    // first band r nb / C <= b
+    };
+    q->shift = 0;
+    for (int sft = 0; sft < ny; ++sft) {
+        bool whole = true;
+        for (const auto &f : span)
+            whole = whole && cta_of((f.second.first - sft + ny) % ny) == cta_of((f.second.second - sft + ny) % ny);
+        if (whole) {
+            q->shift = sft;
+            break;
+        }
+    }
+    // warps whose cells (FP32: with the row above and the column to the left of each thread's block) hold more
+    // than one material keep their coefficients in shared memory (per geometry)
+    const int halo = q->fp64 ? 0 : 1;
+    int cwords = 0, gen_max = 0;
+    res2d_words(q->fp64, q->rb, &cwords);
+    std::map<int, std::vector<int>> gen;
+    auto gen_of = [&](int geo) -> const std::vector<int> & {
+        auto it = gen.find(geo);
+        if (it != gen.end()) return it->second;
+        const std::vector<uint8_t> &mat = D.geos[geo].mat;
+        std::vector<int> g((size_t)q->cluster * nwarp, -1);
+        for (int r = 0; r < q->cluster; ++r) {
+            const int b0 = r * q->nb / q->cluster, b1 = (r + 1) * q->nb / q->cluster;
+            int n = 0;
+            for (int v = 0; v < nwarp; ++v) {
+                int first = -1;
+                bool mixed = false;
+                for (int t = 32 * v; t < 32 * v + 32 && !mixed; ++t) {
+                    const int b = b0 + t / q->tcols, x0 = t % q->tcols * cx;
+                    if (b >= b1) break;
+                    const int y0 = (int)((int64_t)b * ny / q->nb), y1 = (int)((int64_t)(b + 1) * ny / q->nb), x1 = std::min(nx, x0 + cx);
+                    for (int j = y0 - halo; j < y1 && !mixed; ++j)
+                        for (int i = x0 - halo; i < x1; ++i) {
+                            if (j < y0 && i < x0) continue;
+                            const int m = mat[(size_t)((j + q->shift + ny) % ny) * nx + (i < 0 ? nx - 1 : i)];
+                            if (first < 0) first = m;
+                            mixed = mixed || m != first;
+                        }
+                }
+                if (mixed) g[(size_t)r * nwarp + v] = n++;
+            }
+            gen_max = std::max(gen_max, n);
+        }
+        return gen.emplace(geo, std::move(g)).first->second;
+    };
+    std::vector<std::vector<DevEntR>> bucket((size_t)q->cluster);
+    std::vector<DevResWarp> rec((size_t)q->cluster * nwarp);
+    for (const Sim &sm : D.sims) {
+        std::fill(rec.begin(), rec.end(), DevResWarp{});
+        for (auto &b : bucket) b.clear();
+        const int arrays = sm.second_u ? 1 : 2;
+        // the place of an entry: CTA, warp record, lane, row and element of the block
+        auto place = [&](const Entry &e, int *cta, int *lane, int *row, int *el) -> DevResWarp & {
+            const int i = (int)(e.idx % nx), j = (int)((e.idx / nx - q->shift + ny) % ny);   // the cluster's row
+            const int b = (int)(((int64_t)(j + 1) * q->nb - 1) / ny), r = cta_of(j);
+            const int t = (b - (int)((int64_t)r * q->nb / q->cluster)) * q->tcols + i / cx;
+            *cta = r;
+            *lane = t % 32;
+            *row = j - (int)((int64_t)b * ny / q->nb);
+            *el = i % cx;
+            return rec[(size_t)r * nwarp + t / 32];
+        };
+        int cta, lane, row, el;
+        for (const Entry &e : sm.meas) {
+            if (sm.second_u ? e.arr != 0 : (e.arr != 1 && e.arr != 2)) return false;   // the sigma group only
+            DevResWarp &w = place(e, &cta, &lane, &row, &el);
+            w.lanes |= 1u << lane;
+            w.rows |= 1u << row;
+        }
+        const std::vector<int> &g = gen_of(sm.geo);
+        for (int r = 0; r < q->cluster; ++r) {
+            int stage = 0;
+            for (int v = 0; v < nwarp; ++v) {
+                DevResWarp &w = rec[(size_t)r * nwarp + v];
+                w.gen = g[(size_t)r * nwarp + v];
+                w.stride = arrays * __builtin_popcount(w.rows);
+                w.stage0 = stage;
+                stage += __builtin_popcount(w.lanes) * w.stride;
+            }
+            q->stage_words = std::max(q->stage_words, stage);
+        }
+        // an entry's partial sum is its place in its grid row (modulo 32), as in the tiles of the multi-step kernels
+        std::vector<std::pair<int64_t, const Entry *>> order;
+        for (const Entry &e : sm.meas) order.push_back({e.idx, &e});
+        std::stable_sort(order.begin(), order.end(), [](const auto &x, const auto &y) { return x.first < y.first; });
+        int64_t row_at = -1;
+        int place_in_row = 0;
+        for (const auto &oe : order) {
+            const Entry &e = *oe.second;
+            if (e.idx / nx != row_at) {
+                row_at = e.idx / nx;
+                place_in_row = 0;
+            }
+            const int sum = place_in_row++ % 32;
+            const DevResWarp &w = place(e, &cta, &lane, &row, &el);
+            const int word = w.stage0 + __builtin_popcount(w.lanes & ((1u << lane) - 1u)) * w.stride +
+                             __builtin_popcount(w.rows & ((1u << row) - 1u)) * arrays + (sm.second_u ? 0 : e.arr - 1);
+            bucket[cta].push_back(DevEntR{word * cx + el, sum, e.re});
+        }
+        const int64_t e_sim = (int64_t)P->resE.size();
+        for (auto &b : bucket) {
+            if ((int)b.size() > q->threads) return false;
+            q->ne_max = std::max(q->ne_max, (int)b.size());
+            std::stable_sort(b.begin(), b.end(), [](const DevEntR &x, const DevEntR &y) { return x.sum < y.sum; });
+            DevResCta rc{(int)((int64_t)P->resE.size() - e_sim), (int)b.size(), {}};
+            for (int v = 0, k = 0; v <= 32; ++v) {
+                while (k < (int)b.size() && b[k].sum < v) ++k;
+                rc.slot[v] = (short)k;
+            }
+            P->resC.push_back(rc);
+            P->resE.insert(P->resE.end(), b.begin(), b.end());
+        }
+        P->resW.insert(P->resW.end(), rec.begin(), rec.end());
+    }
+    q->gen_words = gen_max * 32 * cwords;
+    q->smem += 16 * (q->gen_words + 2 * q->stage_words) + res2d_proj_bytes(q->fp64, q->ne_max);
+    if (nwarp * 32 * res2d_words(q->fp64, q->rb, &cwords) + q->gen_words + 2 * q->stage_words >= 1 << 16) return false;   // packed into 16 bits
+    return q->smem <= RES_SMEM_MAX;
+}
+
+// allow_resident: the caller left steps_per_launch to the default
+static int prepare_plan(casimir_plan_t *P, bool allow_resident)
 {
     PlanData &D = P->data;
     P->fp64 = D.prob.precision == CASIMIR_FP64;
@@ -135,10 +284,27 @@ static int prepare_plan(casimir_plan_t *P)
             }
         P->pml_off.push_back(po);
     }
+    // 2D TM/TE plans on a device: the first shape of the resident march that holds them
+    if (allow_resident && P->ctx && !D.sims.empty() && D.geos[D.sims[0].geo].family != FAM_FULL &&
+        6 * (int64_t)D.prob.n[0] * D.prob.n[1] < ((int64_t)1 << 31)) {
+        cudaSetDevice(P->ctx->device);
+        for (Res2dShape &q : res2d_shapes(P->fp64, D.prob.n[0], D.prob.n[1], (int)D.sims.size()))
+            if (resident_tables(P, &q)) {
+                P->resident = true;
+                P->res = q;
+                break;
+            }
+        if (!P->resident) {
+            P->resW.clear();
+            P->resC.clear();
+            P->resE.clear();
+        }
+    }
     // sims, tiles, entries, sources
     int64_t off = 0;
     std::map<int, std::vector<int>> march_variants;   // per geometry: kernel variant of each march tile
     std::map<int, std::vector<int>> mar2_variants;    // per geometry: variant of each two-step march tile
+    int64_t rese = 0;                                 // entries of the resident march so far
     for (size_t s = 0; s < D.sims.size(); ++s) {
         const Sim &sm = D.sims[s];
         const Geo &g = D.geos[sm.geo];
@@ -181,9 +347,14 @@ static int prepare_plan(casimir_plan_t *P)
             hs.src0 = (int)P->src.size();
             for (const Entry &e : sm.src) P->src.push_back(DevSrc{hs.field_off + e.arr * N + e.idx, e.re});
             hs.nsrc = (int)P->src.size() - hs.src0;
-            // multi-step tiles: tile_xk(K) wide for K steps per launch, entries sorted by row with
-            // per-row offsets
-            {
+            if (P->resident) {
+                hs.resw0 = (int64_t)s * P->res.cluster * (P->res.threads / 32);
+                hs.resc0 = (int64_t)s * P->res.cluster;
+                hs.rese0 = rese;
+                for (int v = 0; v < P->res.cluster; ++v) rese += P->resC[hs.resc0 + v].ne;
+            } else {
+                // multi-step tiles: tile_xk(K) wide for K steps per launch, entries sorted by row with
+                // per-row offsets
                 const int TXK = tile_xk(P->opts.steps_per_launch == 3 ? 3 : 2);
                 int tx2 = (hs.nx + TXK - 1) / TXK;
                 std::vector<std::vector<std::pair<int, DevEnt>>> b2(tx2 * ty);
@@ -545,11 +716,12 @@ static int prepare_plan(casimir_plan_t *P)
                                align256(P->src.size() * sizeof(DevSrc)) + align256(P->ents6.size() * sizeof(DevEnt6)) +
                                align256(P->src6.size() * sizeof(DevSrc6)) + align256(P->lor_all.size() * 8) +
                                align256(P->pml_all.size() * P->rsize) + align256(P->entsM.size() * sizeof(DevEnt)) +
-                               align256(P->lorc_all.size() * P->rsize));
-    P->request_bytes = (int64_t)(align256(P->field_elems * P->rsize) + 2 * align256(P->sims.size() * 8) +
+                               align256(P->lorc_all.size() * P->rsize) + align256(P->resW.size() * sizeof(DevResWarp)) +
+                               align256(P->resC.size() * sizeof(DevResCta)) + align256(P->resE.size() * sizeof(DevEntR)));
+    P->request_bytes = (int64_t)(align256(P->field_elems * P->rsize) + 2 * align256((P->sims.size() + 1) * 8) +
                                  P->tiles.size() * sizeof(DevTile) + P->tiles6.size() * sizeof(DevTile6) +
                                  P->tiles2.size() * sizeof(DevTile2) + P->tilesM.size() * sizeof(DevTile) +
-                                 P->sims.size() * std::max(sizeof(DevSim2D), sizeof(DevSim6)));
+                                 P->sims.size() * std::max(sizeof(DevRes2D), sizeof(DevSim6)));
     return CASIMIR_OK;
 }
 
@@ -575,13 +747,14 @@ int upload_plan(casimir_plan_t *P, cudaStream_t st)
     NvtxRange nvtx_("casimir.upload");
     if (P->dev.block) return CASIMIR_OK;
     casimir_ctx *c = P->ctx;
-    size_t sz[13] = {align256(P->mat_all.size()), align256(P->coef_all.size() * P->rsize),
+    size_t sz[16] = {align256(P->mat_all.size()), align256(P->coef_all.size() * P->rsize),
                      align256(P->data.gw.size() * 8), align256(P->ents.size() * sizeof(DevEnt)),
                      align256(P->src.size() * sizeof(DevSrc)), align256(P->ents6.size() * sizeof(DevEnt6)),
                      align256(P->src6.size() * sizeof(DevSrc6)), align256(P->lor_all.size() * 8),
                      align256(P->pml_all.size() * P->rsize), align256(P->ents2.size() * sizeof(DevEnt)),
                      align256(P->rowptr2.size() * sizeof(int)), align256(P->entsM.size() * sizeof(DevEnt)),
-                     align256(P->lorc_all.size() * P->rsize)};
+                     align256(P->lorc_all.size() * P->rsize), align256(P->resW.size() * sizeof(DevResWarp)),
+                     align256(P->resC.size() * sizeof(DevResCta)), align256(P->resE.size() * sizeof(DevEntR))};
     size_t total = 0;
     for (size_t q : sz) total += q;
     void *blk;
@@ -602,7 +775,10 @@ int upload_plan(casimir_plan_t *P, cudaStream_t st)
     P->dev.ents2 = (DevEnt *)p; p += sz[9];
     P->dev.rowptr2 = (int *)p; p += sz[10];
     P->dev.entsM = (DevEnt *)p; p += sz[11];
-    P->dev.lorc = p;
+    P->dev.lorc = p; p += sz[12];
+    P->dev.resw = (DevResWarp *)p; p += sz[13];
+    P->dev.resc = (DevResCta *)p; p += sz[14];
+    P->dev.rese = (DevEntR *)p;
     if ((rc = put_table(P->mat_all, P->dev.mat, st))) return rc;
     if ((rc = put_real(P->coef_all, P->dev.coef, P->fp64, st))) return rc;
     if ((rc = put_table(P->data.gw, P->dev.gw, st))) return rc;
@@ -616,6 +792,9 @@ int upload_plan(casimir_plan_t *P, cudaStream_t st)
     if ((rc = put_table(P->rowptr2, P->dev.rowptr2, st))) return rc;
     if ((rc = put_table(P->entsM, P->dev.entsM, st))) return rc;
     if ((rc = put_real(P->lorc_all, P->dev.lorc, P->fp64, st))) return rc;
+    if ((rc = put_table(P->resW, P->dev.resw, st))) return rc;
+    if ((rc = put_table(P->resC, P->dev.resc, st))) return rc;
+    if ((rc = put_table(P->resE, P->dev.rese, st))) return rc;
     c->used += total;
     return CASIMIR_OK;
 }
@@ -635,7 +814,7 @@ static int admit(casimir_ctx *c, casimir_request *r)
     casimir_plan_t *P = r->plan;
     int rc = upload_plan(P, c->stream);
     if (rc) return rc;
-    size_t bf = align256(P->field_elems * P->rsize), ba = align256(P->sims.size() * 8);
+    size_t bf = align256(P->field_elems * P->rsize), ba = align256((P->sims.size() + 1) * 8);   // tail sums, then a status word
     void *blk;
     rc = dev_alloc(c, bf + 2 * ba, &blk);
     if (rc) return rc;
@@ -648,7 +827,7 @@ static int admit(casimir_ctx *c, casimir_request *r)
     launch_inject(P->fp64, blk, P->dev.src, (int)P->src.size(), c->stream);
     launch_inject6(P->fp64, blk, P->dev.src6, (int)P->src6.size(), c->stream);
     CUDA_TRY(cudaGetLastError());
-    if (!r->h_acc) CUDA_TRY(cudaMallocHost((void **)&r->h_acc, std::max<size_t>(1, 2 * P->sims.size()) * 8));
+    if (!r->h_acc) CUDA_TRY(cudaMallocHost((void **)&r->h_acc, (2 * P->sims.size() + 1) * 8));
     // waves of consecutive simulations whose field blocks fit the wave budget
     r->waves.clear();
     r->waves_done = 0;
@@ -822,6 +1001,7 @@ static int rebuild(casimir_ctx *c)
     std::vector<DevTile2> tc2[2];
     std::vector<DevSim6> sm2[2 * MAR2_VARIANTS];    // Cartesian march, two steps per launch
     std::vector<DevTile2> tm2[2 * MAR2_VARIANTS];
+    std::vector<std::pair<Res2dShape, std::vector<DevRes2D>>> res;   // resident 2D runs by shape
     for (auto &aw : c->active_waves) {
         casimir_request *r = aw.first;
         const casimir_request::Wave &w = r->waves[aw.second];
@@ -829,7 +1009,28 @@ static int rebuild(casimir_ctx *c)
         for (size_t s = w.s_begin; s < w.s_end; ++s) {
             const HostSim &hs = P->sims[s];
             char *blk = (char *)r->block;
-            if (!hs.full) {
+            if (P->resident) {
+                const Res2dShape &q = P->res;
+                size_t gi = 0;
+                while (gi < res.size() && !(res[gi].first.fp64 == q.fp64 && res[gi].first.rb == q.rb && res[gi].first.cluster == q.cluster &&
+                                            res[gi].first.threads == q.threads && res[gi].first.smem == q.smem)) ++gi;
+                if (gi == res.size()) res.push_back({q, {}});
+                DevRes2D d{};
+                make_sim2d(P, blk, r->acc, r->tail, w.s0, s, &d.s);
+                d.warps = P->dev.resw + hs.resw0;
+                d.ctas = P->dev.resc + hs.resc0;
+                d.ents = P->dev.rese + hs.rese0;
+                d.status = (int *)(r->tail + P->sims.size());
+                d.gen_words = q.gen_words;
+                d.stage_words = q.stage_words;
+                d.ne_max = q.ne_max;
+                d.shift = q.shift;
+                d.carry_off = (3 * (int64_t)hs.nx * hs.ny * (int64_t)P->rsize + 15) / 16;
+                d.tcols = q.tcols;
+                d.nb = q.nb;
+                d.k = P->k2d;
+                res[gi].second.push_back(d);
+            } else if (!hs.full) {
                 auto &sv = s2[P->fp64];
                 auto &tv = t2[P->fp64];
                 int idx = (int)sv.size();
@@ -981,9 +1182,22 @@ static int rebuild(casimir_ctx *c)
     c->groups[11].ntiles = (int)tt[1].size();
     c->groups[casimir_ctx::G_T3].ntiles = (int)tt[2].size();
     c->groups[casimir_ctx::G_T3 + 1].ntiles = (int)tt[3].size();
+    c->nres = (int)res.size();
+    if (c->res.size() < res.size()) c->res.resize(res.size());
+    for (size_t gi = 0; gi < res.size(); ++gi) {
+        auto &G = c->res[gi];
+        const size_t bytes = res[gi].second.size() * sizeof(DevRes2D);
+        int rc = grow(c, &G.sims, &G.cap, bytes);
+        if (rc) return rc;
+        CUDA_TRY(cudaMemcpyAsync(G.sims, res[gi].second.data(), bytes, cudaMemcpyHostToDevice, c->stream));
+        G.shape = res[gi].first;
+        G.nsims = (int)res[gi].second.size();
+        c->ntiles += G.nsims;
+    }
     CUDA_TRY(cudaStreamSynchronize(c->stream));   // host vectors die here
     drop_graphs(c);
     c->dirty = false;
+    c->index_ms = 0;   // another set of runs
     return CASIMIR_OK;
 }
 
@@ -1031,27 +1245,45 @@ static void launch_unit(casimir_ctx *c, int gi, int j, cudaStream_t st)
 // Launch k consecutive steps.  The units of one step touch disjoint tiles and read only the
 // previous step's buffers, so with more than one unit they run side by side on auxiliary
 // streams (forked from and joined back into the context's stream every step), which lets one
-// unit's last partial wave overlap the next unit.
+// unit's last partial wave overlap the next unit.  Resident groups run all k launch indices in one
+// launch, beside the others on the last auxiliary streams.
 static void launch_steps(casimir_ctx *c, int k)
 {
     static const bool no_fork = std::getenv("CASIMIR_NO_FORK") != nullptr;
     int units[casimir_ctx::NGROUPS], nu = 0;
     for (int gi = 0; gi < casimir_ctx::NGROUPS; ++gi)
         if (c->groups[gi].ntiles > 0) units[nu++] = gi;
+    auto resident = [&](int q, cudaStream_t st) {
+        launch_res2d(c->res[q].shape, (const DevRes2D *)c->res[q].sims, c->res[q].nsims, c->d_launch, 0, k, st);
+    };
+    const bool beside = nu + c->nres > 1 && !no_fork;
+    const int nra = beside ? std::min(c->nres, casimir_ctx::NAUX / 2) : 0;   // streams of the resident groups
+    if (nra > 0) {
+        cudaEventRecord(c->ev_fork, c->stream);
+        for (int q = 0; q < nra; ++q) cudaStreamWaitEvent(c->aux[casimir_ctx::NAUX - 1 - q], c->ev_fork, 0);
+        for (int q = 0; q < c->nres; ++q) resident(q, c->aux[casimir_ctx::NAUX - 1 - q % nra]);
+    } else {
+        for (int q = 0; q < c->nres; ++q) resident(q, c->stream);
+    }
     const bool fork = nu > 1 && !no_fork;
-    for (int j = 0; j < k; ++j) {
+    for (int j = 0; j < k && nu > 0; ++j) {
         if (!fork) {
             for (int u = 0; u < nu; ++u) launch_unit(c, units[u], j, c->stream);
             continue;
         }
         cudaEventRecord(c->ev_fork, c->stream);
-        const int na = std::min(nu, casimir_ctx::NAUX);
+        const int na = std::min(nu, casimir_ctx::NAUX - nra);
         for (int a = 0; a < na; ++a) cudaStreamWaitEvent(c->aux[a], c->ev_fork, 0);
         for (int u = 0; u < nu; ++u) launch_unit(c, units[u], j, c->aux[u % na]);
         for (int a = 0; a < na; ++a) {
             cudaEventRecord(c->ev_join[a], c->aux[a]);
             cudaStreamWaitEvent(c->stream, c->ev_join[a], 0);
         }
+    }
+    for (int q = 0; q < nra; ++q) {
+        const int a = casimir_ctx::NAUX - 1 - q;
+        cudaEventRecord(c->ev_join[a], c->aux[a]);
+        cudaStreamWaitEvent(c->stream, c->ev_join[a], 0);
     }
     launch_bump(c->d_launch, k, c->stream);
 }
@@ -1093,7 +1325,7 @@ static int run_chunk(casimir_ctx *c, int k)
     for (int gi = 0; gi < casimir_ctx::NGROUPS; ++gi)
         if (c->groups[gi].ntiles > 0)
             per_step += ((gi >= 2 && gi < 10) || (gi >= casimir_ctx::G_LINE3 && gi < casimir_ctx::G_CYL)) ? 2 : 1;
-    for (casimir_request *r : c->active) r->launches += (int64_t)k * per_step + 1;
+    for (casimir_request *r : c->active) r->launches += (int64_t)k * per_step + c->nres + 1;
     return CASIMIR_OK;
 }
 
@@ -1117,12 +1349,24 @@ static void finish_request(casimir_ctx *c, casimir_request *r, int status)
     r->F[D.prob.force_axis] = s;
     r->err = te;
     dev_free(c, r->block);
-    c->used -= align256(P->field_elems * P->rsize) + 2 * align256(ns * 8);
+    c->used -= align256(P->field_elems * P->rsize) + 2 * align256((ns + 1) * 8);
     r->block = nullptr;
     r->t_done = now_ms();
+    if (status == CASIMIR_OK && *(const int *)(r->h_acc + 2 * ns)) {   // a resident cluster's wait ran out
+        status = CASIMIR_ECUDA;
+        r->msg = "resident march: a wait between the CTAs of a cluster ran out";
+    }
     r->status = status;
     P->inflight--;
     r->state.store(status == CASIMIR_OK ? 2 : 3, std::memory_order_release);
+}
+
+// Whether every active run is on the resident march.
+static bool only_resident(const casimir_ctx *c)
+{
+    for (const auto &G : c->groups)
+        if (G.ntiles > 0) return false;
+    return c->nres > 0;
 }
 
 // One engine iteration: run a chunk, then issue copy-backs for finished requests
@@ -1143,14 +1387,24 @@ static int engine_iterate(casimir_ctx *c)
         }
         if (rem > 0) {
             int k = (int)std::min<int64_t>(64, rem);
+            const double wd = c->watchdog_ms.load();
+            if (wd > 0 && only_resident(c)) {
+                // the watchdog is checked between chunks: a resident chunk is one launch of up to 192 steps over
+                // every simulation, so it is cut to about a thousandth of the limit (a power of two indices)
+                int cut = 8;
+                if (c->index_ms > 0)
+                    for (cut = 1; cut < 64 && 2 * cut * c->index_ms <= 1e-3 * wd;) cut *= 2;
+                k = std::min(k, cut);
+            }
             int rc = run_chunk(c, k);
             if (rc) return rc;
             CUDA_TRY(cudaEventSynchronize(c->ev1));
             float ms = 0;
             cudaEventElapsedTime(&ms, c->ev0, c->ev1);
+            c->index_ms = ms / k;
             std::lock_guard<std::mutex> lk(c->mu);   // the statistics are read under the lock
             c->step_ms += ms;
-            c->step_launches += k;
+            c->step_launches += only_resident(c) ? c->nres : k;   // one per index, or per chunk where every run is resident
             for (auto &aw : c->active_waves) {
                 const casimir_request::Wave &w = aw.first->waves[aw.second];
                 const casimir_plan_t *P = aw.first->plan;
@@ -1184,7 +1438,7 @@ static int engine_iterate(casimir_ctx *c)
             if (!done) drop_waves(c, r);
             size_t ns = r->plan->sims.size();
             CUDA_TRY(cudaMemcpyAsync(r->h_acc, r->acc, ns * 8, cudaMemcpyDeviceToHost, c->stream));
-            CUDA_TRY(cudaMemcpyAsync(r->h_acc + ns, r->tail, ns * 8, cudaMemcpyDeviceToHost, c->stream));
+            CUDA_TRY(cudaMemcpyAsync(r->h_acc + ns, r->tail, (ns + 1) * 8, cudaMemcpyDeviceToHost, c->stream));
             if (!r->done_ev) CUDA_TRY(cudaEventCreateWithFlags(&r->done_ev, cudaEventDisableTiming));
             CUDA_TRY(cudaEventRecord(r->done_ev, c->stream));
             r->copy_issued = true;
@@ -1285,6 +1539,7 @@ int casimir_ctx_create(int device, uint64_t budget, casimir_ctx_t **out)
     if (device < 0 || device >= ndev) return fail(CASIMIR_EINVAL, "no such CUDA device");
     CUDA_TRY(cudaSetDevice(device));
     CUDA_TRY(march6_prepare());
+    CUDA_TRY(res2d_prepare());
     auto *c = new casimir_ctx();
     c->device = device;
     size_t fr = 0, tot = 0;
@@ -1326,6 +1581,7 @@ void casimir_ctx_destroy(casimir_ctx_t *c)
         dev_free(c, G.sims);
         dev_free(c, G.tiles);
     }
+    for (auto &G : c->res) dev_free(c, G.sims);
     cudaFree(c->d_launch);
     cudaEventDestroy(c->ev0);
     cudaEventDestroy(c->ev1);
@@ -1360,7 +1616,7 @@ int casimir_ctx_set_allocator(casimir_ctx_t *c, casimir_alloc_fn a, casimir_free
 {
     if (!c || (!a) != (!f)) return fail(CASIMIR_EINVAL, "allocator needs both callbacks");
     std::lock_guard<std::mutex> lk(c->mu);
-    if (!c->active.empty() || !c->queue.empty() || c->groups[0].sims) return fail(CASIMIR_EBUSY, "set the allocator before the first request");
+    if (!c->active.empty() || !c->queue.empty() || c->groups[0].sims || !c->res.empty()) return fail(CASIMIR_EBUSY, "set the allocator before the first request");
     c->alloc = a;
     c->freef = f;
     c->user = user;
@@ -1449,10 +1705,13 @@ static int make_plan(casimir_ctx_t *c, const casimir_problem *p, const casimir_p
     P->ctx = c;
     int rc = resolve_options(opts, &P->opts, p->precision == CASIMIR_FP64, has_pml3d(*p));
     if (rc) { delete P; return rc; }
+    // a number of time steps per launch, asked for in the options or by the environment, names a
+    // kernel of that many; the default leaves 2D TM/TE runs to the resident march where it fits
+    const bool resident = (!opts || opts->steps_per_launch == 0) && !std::getenv("CASIMIR_STEP2D_K");
     std::string err;
     rc = build_plan(p, &P->data, &err);
     if (rc) { delete P; return fail(rc, err); }
-    rc = prepare_plan(P);
+    rc = prepare_plan(P, resident);
     if (rc) { delete P; return rc; }
     if (c && (uint64_t)(P->table_bytes + P->request_bytes) > c->budget) {
         delete P;
@@ -1507,8 +1766,8 @@ static casimir_plan_options autotune(casimir_ctx *c, const casimir_problem &p)
             cand.push_back(o);
         }
     } else {
-        // the default first (ties keep it), then the other fusion depths
-        cand = {dflt};
+        // the default first (ties keep it: the resident march where it fits), then the fusion depths
+        cand = {casimir_plan_options{}, dflt};
         for (int k : {3, 2, 1})
             if (k != dflt.steps_per_launch) {
                 casimir_plan_options o = dflt;
@@ -1521,7 +1780,7 @@ static casimir_plan_options autotune(casimir_ctx *c, const casimir_problem &p)
         std::lock_guard<std::mutex> lk(c->mu);
         auto it = c->tuned.find(key);
         if (it != c->tuned.end()) return it->second;
-        if (!c->active.empty() || !c->queue.empty() || c->sync_busy) return dflt;   // never disturb running work
+        if (!c->active.empty() || !c->queue.empty() || c->sync_busy) return casimir_plan_options{};   // never disturb running work
     }
     casimir_problem trial = p;
     trial.n_steps = std::min(p.n_steps, 128);
@@ -1529,7 +1788,7 @@ static casimir_plan_options autotune(casimir_ctx *c, const casimir_problem &p)
     const double ms0 = c->step_ms;
     const int64_t l0 = c->step_launches, cu0 = c->cell_updates;
     double best_t = 0;
-    casimir_plan_options best = dflt;
+    casimir_plan_options best{};
     bool any = false;
     for (const casimir_plan_options &o : cand) {
         casimir_plan_t *tp = nullptr;
@@ -1834,6 +2093,7 @@ int casimir_run(casimir_plan_t *P, double F[3], double *per_sim, casimir_stats *
         c->pending_waves.clear();
         c->active_bytes = 0;
         c->dirty = true;
+        P->inflight--;   // the plan can be destroyed
     }
     c->sync_busy = 0;
     int status = rc ? rc : r.status.load();

@@ -62,6 +62,7 @@ struct HostSim {
     int tile2_0, ntile2;   // range in the plan's two-step tile list (2D)
     int ent0, nent;        // range in the plan's entry list (bucketed by tile)
     int src0, nsrc;        // range in the plan's source list
+    int64_t resw0 = 0, resc0 = 0, rese0 = 0;   // resident runs: first warp record, CTA record and entry of the simulation
 };
 
 struct HostTile {
@@ -92,6 +93,9 @@ struct DevPlan {           // device copies of a plan's static tables (kept whil
     DevSrc6 *src6 = nullptr;
     DevEnt *ents2 = nullptr;
     int *rowptr2 = nullptr;
+    DevResWarp *resw = nullptr;
+    DevResCta *resc = nullptr;
+    DevEntR *rese = nullptr;
     double *lor = nullptr;
     void *lorc = nullptr;
     void *pml = nullptr;
@@ -120,6 +124,11 @@ struct casimir_plan {
     std::vector<int> rowptr2;
     int64_t launches = 0;             // launches a request needs (ceil(T/k2d))
     int k2d = 1;                      // time steps per launch of the 2D kernel (1, 2 or 3)
+    bool resident = false;            // 2D TM/TE plan on the resident march
+    Res2dShape res{};
+    std::vector<DevResWarp> resW;     // per simulation, [cluster rank][warp]
+    std::vector<DevResCta> resC;      // per simulation, [cluster rank]
+    std::vector<DevEntR> resE;
     std::vector<HostTile6> tiles6;
     std::vector<HostTile> tilesM;     // march kernel strip tiles (MARCH_W x MARCH_H) with their entries
     std::vector<DevEnt> entsM;
@@ -204,6 +213,16 @@ struct casimir_ctx {
         int ntiles = 0;
     } groups[NGROUPS];
     int ntiles = 0;                   // over all groups
+    // resident 2D runs: one launch per chunk and shape (buffers are reused from batch to batch)
+    struct ResGroup {
+        Res2dShape shape{};
+        void *sims = nullptr;
+        size_t cap = 0;
+        int nsims = 0;
+    };
+    std::vector<ResGroup> res;
+    int nres = 0;                     // groups in use
+    double index_ms = 0;              // time of a launch index in the last chunk
     // waves: simulations are activated in groups whose field bytes fit `wave_bytes`
     // (0: a whole request at once), so that the active working set can stay in L2
     std::atomic<int64_t> wave_bytes{0};

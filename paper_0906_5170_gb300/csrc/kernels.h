@@ -3,6 +3,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include <vector>
+
 namespace cas {
 
 constexpr int TILE_X = 120;   // four warp strips of 30 interior columns
@@ -189,6 +191,51 @@ void launch_march6_cyl2(int fp64, const DevSim6 *sims, const DevTile2 *tiles, in
 constexpr int MAR2_VARIANTS = 4;
 void launch_march6_2(int cplx, int variant, const DevSim6 *sims, const DevTile2 *tiles, int ntiles,
                      const int64_t *launch_base, int64_t launch_add, cudaStream_t st);
+
+// Resident march of the 2D TM/TE simulations (res2d.cu): one cluster of `cluster` CTAs per
+// simulation, fields in registers (in buffer 0 between launches), `count` launch indices of `k` time
+// steps each per launch.
+struct DevResWarp {        // the rows a warp stages for the surface functional (lanes 0: none)
+    unsigned lanes, rows;  // staging lanes, rows of the block that are staged
+    int stage0, stride;    // 16-byte words: the warp's first, and per staging lane
+    int gen, pad;          // -1: all its cells are of one material; else its place among those that are not
+};
+struct DevResCta {         // the functional's entries of one CTA, one per thread, by partial sum
+    int e0, ne;
+    short slot[34];        // first entry of partial sum q, q = 0 .. 32
+};
+struct DevEntR {
+    int off;               // element within the CTA's staged rows
+    int sum;               // its partial sum, 0 .. 31
+    double w;
+};
+struct DevRes2D {
+    DevSim2D s;
+    const DevResWarp *warps;   // [cluster rank][warp]
+    const DevResCta *ctas;     // [cluster rank]
+    const DevEntR *ents;
+    int *status;               // set when a wait ran out
+    int64_t carry_off;         // the CTAs' sums between launches, in 16-byte pairs from s.fields
+    int tcols, nb, k;          // threads per row band, row bands, time steps per launch index
+    int gen_words;             // 16-byte words of coefficients behind the slots
+    int stage_words;           // and of one buffer of staged rows behind them (then the launch's weights)
+    int ne_max;                // entries of a CTA at most
+    int shift, pad;            // grid row of the cluster's first row (the grid is a torus)
+};
+struct Res2dShape {
+    int fp64, rb;          // rows of a thread's block
+    int cluster, threads, smem;
+    int tcols, nb;
+    int gen_words, stage_words, ne_max, shift;
+};
+int res2d_words(int fp64, int rb, int *coef);   // 16-byte words of a thread's slots, and of its coefficients
+constexpr int RES_CLUSTER_MAX = 16;
+constexpr int RES_SMEM_MAX = 226 * 1024;      // dynamic shared memory of a CTA (the rest is static)
+constexpr int RES_LAUNCH_STEPS = 192;         // time steps of one launch at most (its weights sit in shared memory)
+cudaError_t res2d_prepare();
+int res2d_proj_bytes(int fp64, int ne);      // shared memory of the projection's history and sums, ne entries a CTA
+std::vector<Res2dShape> res2d_shapes(int fp64, int nx, int ny, int nsims);
+void launch_res2d(const Res2dShape &q, const DevRes2D *sims, int nsims, const int64_t *launch_base, int64_t launch_add, int count, cudaStream_t st);
 
 void launch_step2d(int fp64, const DevSim2D *sims, const DevTile *tiles, int ntiles,
                    const int64_t *launch_base, int64_t launch_add, cudaStream_t st);
