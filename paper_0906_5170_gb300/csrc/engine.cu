@@ -83,18 +83,19 @@ void dev_free(casimir_ctx *c, void *p)
 
 // Entry tables of a 2D TM/TE plan for the resident march of shape q: the rows each warp of a simulation's
 // cluster stages, and the entries of each CTA, one per thread.  False when the shape cannot hold them
-// (more entries than threads in a CTA, staged rows and coefficients beyond the shared memory left, or sums beyond the second
-// field buffer, where they wait between launches).
+// (more entries than threads in a CTA, staged rows and coefficients beyond the shared memory left, or more pieces than
+// the second field buffer holds the terms of).
 static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
 {
     const PlanData &D = P->data;
     const int cx = q->fp64 ? 2 : 4, nwarp = q->threads / 32, nx = D.prob.n[0], ny = D.prob.n[1];
-    const int64_t N = (int64_t)nx * ny;
     P->resW.clear();
     P->resC.clear();
     P->resE.clear();
-    q->stage_words = q->ne_max = 0;
-    if ((int64_t)q->cluster * 16 + 16 > 3 * N * (int64_t)P->rsize) return false;
+    P->resT.clear();
+    P->resNT.clear();
+    q->stage_words = q->ne_max = q->np_max = q->npiece_max = q->ntile_max = 0;
+    const int txk = tile_xk(P->opts.steps_per_launch == 3 ? 3 : 2), tx = (nx + txk - 1) / txk;   // tiles of the multi-step kernels
     // the cluster's first row: the first that leaves the rows of every horizontal face in one CTA
     std::map<int, std::pair<int, int>> span;   // face -> its measured rows
     for (const Sim &sm : D.sims)
@@ -154,11 +155,9 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
         }
         return gen.emplace(geo, std::move(g)).first->second;
     };
-    std::vector<std::vector<DevEntR>> bucket((size_t)q->cluster);
     std::vector<DevResWarp> rec((size_t)q->cluster * nwarp);
     for (const Sim &sm : D.sims) {
         std::fill(rec.begin(), rec.end(), DevResWarp{});
-        for (auto &b : bucket) b.clear();
         const int arrays = sm.second_u ? 1 : 2;
         // the place of an entry: CTA, warp record, lane, row and element of the block
         auto place = [&](const Entry &e, int *cta, int *lane, int *row, int *el) -> DevResWarp & {
@@ -190,41 +189,78 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
             }
             q->stage_words = std::max(q->stage_words, stage);
         }
-        // an entry's partial sum is its place in its grid row (modulo 32), as in the tiles of the multi-step kernels
+        // on a horizontal face an entry's partial sum is its place in its grid row (modulo 32), as in the tiles of
+        // the multi-step kernels; elsewhere the entries are dealt to the first 16 in turn
         std::vector<std::pair<int64_t, const Entry *>> order;
         for (const Entry &e : sm.meas) order.push_back({e.idx, &e});
         std::stable_sort(order.begin(), order.end(), [](const auto &x, const auto &y) { return x.first < y.first; });
         int64_t row_at = -1;
         int place_in_row = 0;
+        std::vector<std::vector<std::pair<int, DevEntR>>> byp((size_t)q->cluster);   // per CTA: (tile, entry)
+        std::map<std::pair<int, int>, int> pieces;                                   // (tile, CTA) -> number
         for (const auto &oe : order) {
             const Entry &e = *oe.second;
-            if (e.idx / nx != row_at) {
-                row_at = e.idx / nx;
+            const int ti = (int)(e.idx % nx) / txk, tile = (int)(e.idx / nx) / TILE_Y * tx + ti;
+            const int64_t at = e.idx / nx * tx + ti;   // the row of the tile
+            if (at != row_at && D.faces[sm.face].axis == 1) {
+                row_at = at;
                 place_in_row = 0;
             }
-            const int sum = place_in_row++ % 32;
+            const int sum = place_in_row++ % (D.faces[sm.face].axis == 1 ? 32 : 16);
             const DevResWarp &w = place(e, &cta, &lane, &row, &el);
             const int word = w.stage0 + __builtin_popcount(w.lanes & ((1u << lane) - 1u)) * w.stride +
                              __builtin_popcount(w.rows & ((1u << row) - 1u)) * arrays + (sm.second_u ? 0 : e.arr - 1);
-            bucket[cta].push_back(DevEntR{word * cx + el, sum, e.re});
+            byp[cta].push_back({tile, DevEntR{word * cx + el, sum, e.re}});
+            pieces[{tile, cta}] = 0;
         }
+        short tp[RES_TILES + 1] = {};
+        int npiece = 0, ntile = 0, last_tile = -1;
+        for (auto &pe : pieces) {   // by tile, then CTA
+            if (pe.first.first != last_tile) {
+                if (ntile == RES_TILES) return false;
+                tp[ntile++] = (short)npiece;
+                last_tile = pe.first.first;
+            }
+            pe.second = npiece++;
+        }
+        tp[ntile] = (short)npiece;
+        q->npiece_max = std::max(q->npiece_max, npiece);
+        q->ntile_max = std::max(q->ntile_max, ntile);
+        P->resT.insert(P->resT.end(), tp, tp + RES_TILES + 1);
+        P->resNT.push_back(ntile);
         const int64_t e_sim = (int64_t)P->resE.size();
-        for (auto &b : bucket) {
+        for (int r = 0; r < q->cluster; ++r) {
+            auto &b = byp[r];
             if ((int)b.size() > q->threads) return false;
             q->ne_max = std::max(q->ne_max, (int)b.size());
-            std::stable_sort(b.begin(), b.end(), [](const DevEntR &x, const DevEntR &y) { return x.sum < y.sum; });
-            DevResCta rc{(int)((int64_t)P->resE.size() - e_sim), (int)b.size(), {}};
-            for (int v = 0, k = 0; v <= 32; ++v) {
-                while (k < (int)b.size() && b[k].sum < v) ++k;
-                rc.slot[v] = (short)k;
+            std::stable_sort(b.begin(), b.end(), [](const auto &x, const auto &y) {
+                return x.first != y.first ? x.first < y.first : x.second.sum < y.second.sum;
+            });
+            DevResCta rc{};
+            rc.e0 = (int)((int64_t)P->resE.size() - e_sim);
+            rc.ne = (int)b.size();
+            rc.rounded = D.faces[sm.face].axis == 1;
+            for (int k = 0; k < (int)b.size();) {
+                if (rc.np == RES_PIECES) return false;
+                const int tile = b[k].first;
+                rc.piece[rc.np] = (short)pieces[{tile, r}];
+                for (int v = 0; v < 32; ++v) {
+                    while (k < (int)b.size() && b[k].first == tile && b[k].second.sum < v) ++k;
+                    rc.slot[rc.np * 32 + v] = (short)k;
+                }
+                while (k < (int)b.size() && b[k].first == tile) ++k;
+                ++rc.np;
+                rc.slot[rc.np * 32] = (short)k;
             }
+            q->np_max = std::max(q->np_max, (int)rc.np);
             P->resC.push_back(rc);
-            P->resE.insert(P->resE.end(), b.begin(), b.end());
+            for (const auto &be : b) P->resE.push_back(be.second);
         }
         P->resW.insert(P->resW.end(), rec.begin(), rec.end());
     }
+    if ((int64_t)q->npiece_max * RES_LAUNCH_STEPS * 8 + 8 > 3 * (int64_t)nx * ny * (int64_t)P->rsize) return false;   // their terms wait in the second field buffer
     q->gen_words = gen_max * 32 * cwords;
-    q->smem += 16 * (q->gen_words + 2 * q->stage_words) + res2d_proj_bytes(q->fp64, q->ne_max);
+    q->smem += 16 * (q->gen_words + 2 * q->stage_words) + res2d_proj_bytes(*q);
     if (nwarp * 32 * res2d_words(q->fp64, q->rb, &cwords) + q->gen_words + 2 * q->stage_words >= 1 << 16) return false;   // packed into 16 bits
     return q->smem <= RES_SMEM_MAX;
 }
@@ -298,6 +334,7 @@ static int prepare_plan(casimir_plan_t *P, bool allow_resident)
             P->resW.clear();
             P->resC.clear();
             P->resE.clear();
+            P->resT.clear();
         }
     }
     // sims, tiles, entries, sources
@@ -717,7 +754,8 @@ static int prepare_plan(casimir_plan_t *P, bool allow_resident)
                                align256(P->src6.size() * sizeof(DevSrc6)) + align256(P->lor_all.size() * 8) +
                                align256(P->pml_all.size() * P->rsize) + align256(P->entsM.size() * sizeof(DevEnt)) +
                                align256(P->lorc_all.size() * P->rsize) + align256(P->resW.size() * sizeof(DevResWarp)) +
-                               align256(P->resC.size() * sizeof(DevResCta)) + align256(P->resE.size() * sizeof(DevEntR)));
+                               align256(P->resC.size() * sizeof(DevResCta)) + align256(P->resE.size() * sizeof(DevEntR)) +
+                               align256(P->resT.size() * sizeof(short)));
     P->request_bytes = (int64_t)(align256(P->field_elems * P->rsize) + 2 * align256((P->sims.size() + 1) * 8) +
                                  P->tiles.size() * sizeof(DevTile) + P->tiles6.size() * sizeof(DevTile6) +
                                  P->tiles2.size() * sizeof(DevTile2) + P->tilesM.size() * sizeof(DevTile) +
@@ -747,14 +785,15 @@ int upload_plan(casimir_plan_t *P, cudaStream_t st)
     NvtxRange nvtx_("casimir.upload");
     if (P->dev.block) return CASIMIR_OK;
     casimir_ctx *c = P->ctx;
-    size_t sz[16] = {align256(P->mat_all.size()), align256(P->coef_all.size() * P->rsize),
+    size_t sz[17] = {align256(P->mat_all.size()), align256(P->coef_all.size() * P->rsize),
                      align256(P->data.gw.size() * 8), align256(P->ents.size() * sizeof(DevEnt)),
                      align256(P->src.size() * sizeof(DevSrc)), align256(P->ents6.size() * sizeof(DevEnt6)),
                      align256(P->src6.size() * sizeof(DevSrc6)), align256(P->lor_all.size() * 8),
                      align256(P->pml_all.size() * P->rsize), align256(P->ents2.size() * sizeof(DevEnt)),
                      align256(P->rowptr2.size() * sizeof(int)), align256(P->entsM.size() * sizeof(DevEnt)),
                      align256(P->lorc_all.size() * P->rsize), align256(P->resW.size() * sizeof(DevResWarp)),
-                     align256(P->resC.size() * sizeof(DevResCta)), align256(P->resE.size() * sizeof(DevEntR))};
+                     align256(P->resC.size() * sizeof(DevResCta)), align256(P->resE.size() * sizeof(DevEntR)),
+                     align256(P->resT.size() * sizeof(short))};
     size_t total = 0;
     for (size_t q : sz) total += q;
     void *blk;
@@ -778,7 +817,8 @@ int upload_plan(casimir_plan_t *P, cudaStream_t st)
     P->dev.lorc = p; p += sz[12];
     P->dev.resw = (DevResWarp *)p; p += sz[13];
     P->dev.resc = (DevResCta *)p; p += sz[14];
-    P->dev.rese = (DevEntR *)p;
+    P->dev.rese = (DevEntR *)p; p += sz[15];
+    P->dev.rest = (short *)p;
     if ((rc = put_table(P->mat_all, P->dev.mat, st))) return rc;
     if ((rc = put_real(P->coef_all, P->dev.coef, P->fp64, st))) return rc;
     if ((rc = put_table(P->data.gw, P->dev.gw, st))) return rc;
@@ -795,6 +835,7 @@ int upload_plan(casimir_plan_t *P, cudaStream_t st)
     if ((rc = put_table(P->resW, P->dev.resw, st))) return rc;
     if ((rc = put_table(P->resC, P->dev.resc, st))) return rc;
     if ((rc = put_table(P->resE, P->dev.rese, st))) return rc;
+    if ((rc = put_table(P->resT, P->dev.rest, st))) return rc;
     c->used += total;
     return CASIMIR_OK;
 }
@@ -807,6 +848,41 @@ static void drop_graphs(casimir_ctx *c)
 {
     for (auto &kv : c->graphs) cudaGraphExecDestroy(kv.second);
     c->graphs.clear();
+}
+
+// Pinned result buffer of a request: one that a finished request left, or a new one.
+static int take_pinned(casimir_ctx *c, size_t need, casimir_request *r)
+{
+    {
+        std::lock_guard<std::mutex> lk(c->pinned_mu);
+        for (auto &sp : c->pinned)
+            if (sp.first && sp.second >= need) {
+                r->h_acc = sp.first;
+                r->h_bytes = sp.second;
+                sp.first = nullptr;
+                return CASIMIR_OK;
+            }
+    }
+    CUDA_TRY(cudaMallocHost((void **)&r->h_acc, need));
+    r->h_bytes = need;
+    return CASIMIR_OK;
+}
+
+// Leaves it to the next request, or frees it (a large one, or when enough are kept).
+static void give_pinned(casimir_ctx *c, casimir_request *r)
+{
+    if (!r->h_acc) return;
+    if (r->h_bytes <= casimir_ctx::PINNED_MAX) {
+        std::lock_guard<std::mutex> lk(c->pinned_mu);
+        for (auto &sp : c->pinned)
+            if (!sp.first) {
+                sp = {r->h_acc, r->h_bytes};
+                r->h_acc = nullptr;
+                return;
+            }
+    }
+    cudaFreeHost(r->h_acc);
+    r->h_acc = nullptr;
 }
 
 static int admit(casimir_ctx *c, casimir_request *r)
@@ -827,7 +903,10 @@ static int admit(casimir_ctx *c, casimir_request *r)
     launch_inject(P->fp64, blk, P->dev.src, (int)P->src.size(), c->stream);
     launch_inject6(P->fp64, blk, P->dev.src6, (int)P->src6.size(), c->stream);
     CUDA_TRY(cudaGetLastError());
-    if (!r->h_acc) CUDA_TRY(cudaMallocHost((void **)&r->h_acc, (2 * P->sims.size() + 1) * 8));
+    if (!r->h_acc) {
+        rc = take_pinned(c, (2 * P->sims.size() + 1) * 8, r);
+        if (rc) return rc;
+    }
     // waves of consecutive simulations whose field blocks fit the wave budget
     r->waves.clear();
     r->waves_done = 0;
@@ -1025,7 +1104,11 @@ static int rebuild(casimir_ctx *c)
                 d.stage_words = q.stage_words;
                 d.ne_max = q.ne_max;
                 d.shift = q.shift;
-                d.carry_off = (3 * (int64_t)hs.nx * hs.ny * (int64_t)P->rsize + 15) / 16;
+                d.tile_pieces = P->dev.rest + s * (RES_TILES + 1);
+                d.ntile = P->resNT[s];
+                d.np_max = q.np_max;
+                d.term_off = (3 * (int64_t)hs.nx * hs.ny * (int64_t)P->rsize + 7) / 8;   // the second field buffer
+                d.ntile_max = q.ntile_max;
                 d.tcols = q.tcols;
                 d.nb = q.nb;
                 d.k = P->k2d;
@@ -1194,6 +1277,8 @@ static int rebuild(casimir_ctx *c)
         G.nsims = (int)res[gi].second.size();
         c->ntiles += G.nsims;
     }
+    // the launch counter of the step kernels (resident runs take the index from the host)
+    CUDA_TRY(cudaMemcpyAsync(c->d_launch, &c->h_launch, sizeof(int64_t), cudaMemcpyHostToDevice, c->stream));
     CUDA_TRY(cudaStreamSynchronize(c->stream));   // host vectors die here
     drop_graphs(c);
     c->dirty = false;
@@ -1245,34 +1330,21 @@ static void launch_unit(casimir_ctx *c, int gi, int j, cudaStream_t st)
 // Launch k consecutive steps.  The units of one step touch disjoint tiles and read only the
 // previous step's buffers, so with more than one unit they run side by side on auxiliary
 // streams (forked from and joined back into the context's stream every step), which lets one
-// unit's last partial wave overlap the next unit.  Resident groups run all k launch indices in one
-// launch, beside the others on the last auxiliary streams.
-static void launch_steps(casimir_ctx *c, int k)
+// unit's last partial wave overlap the next unit.  `keep` auxiliary streams are left alone.
+static void launch_steps(casimir_ctx *c, int k, int keep)
 {
     static const bool no_fork = std::getenv("CASIMIR_NO_FORK") != nullptr;
     int units[casimir_ctx::NGROUPS], nu = 0;
     for (int gi = 0; gi < casimir_ctx::NGROUPS; ++gi)
         if (c->groups[gi].ntiles > 0) units[nu++] = gi;
-    auto resident = [&](int q, cudaStream_t st) {
-        launch_res2d(c->res[q].shape, (const DevRes2D *)c->res[q].sims, c->res[q].nsims, c->d_launch, 0, k, st);
-    };
-    const bool beside = nu + c->nres > 1 && !no_fork;
-    const int nra = beside ? std::min(c->nres, casimir_ctx::NAUX / 2) : 0;   // streams of the resident groups
-    if (nra > 0) {
-        cudaEventRecord(c->ev_fork, c->stream);
-        for (int q = 0; q < nra; ++q) cudaStreamWaitEvent(c->aux[casimir_ctx::NAUX - 1 - q], c->ev_fork, 0);
-        for (int q = 0; q < c->nres; ++q) resident(q, c->aux[casimir_ctx::NAUX - 1 - q % nra]);
-    } else {
-        for (int q = 0; q < c->nres; ++q) resident(q, c->stream);
-    }
     const bool fork = nu > 1 && !no_fork;
-    for (int j = 0; j < k && nu > 0; ++j) {
+    for (int j = 0; j < k; ++j) {
         if (!fork) {
             for (int u = 0; u < nu; ++u) launch_unit(c, units[u], j, c->stream);
             continue;
         }
         cudaEventRecord(c->ev_fork, c->stream);
-        const int na = std::min(nu, casimir_ctx::NAUX - nra);
+        const int na = std::min(nu, casimir_ctx::NAUX - keep);
         for (int a = 0; a < na; ++a) cudaStreamWaitEvent(c->aux[a], c->ev_fork, 0);
         for (int u = 0; u < nu; ++u) launch_unit(c, units[u], j, c->aux[u % na]);
         for (int a = 0; a < na; ++a) {
@@ -1280,33 +1352,18 @@ static void launch_steps(casimir_ctx *c, int k)
             cudaStreamWaitEvent(c->stream, c->ev_join[a], 0);
         }
     }
-    for (int q = 0; q < nra; ++q) {
-        const int a = casimir_ctx::NAUX - 1 - q;
-        cudaEventRecord(c->ev_join[a], c->aux[a]);
-        cudaStreamWaitEvent(c->stream, c->ev_join[a], 0);
-    }
     launch_bump(c->d_launch, k, c->stream);
 }
 
-// Launch `k` consecutive steps (as a cached CUDA graph, or directly when the
-// environment sets CASIMIR_NO_GRAPHS, e.g. for kernel profiling) and advance
-// the launch counter.
-static int run_chunk(casimir_ctx *c, int k)
+// The graph of k launch indices of the current active set, captured at its first use.
+static int graph_of(casimir_ctx *c, int k, cudaGraphExec_t *out)
 {
-    NvtxRange nvtx_("casimir.chunk");
-    static const bool no_graphs = std::getenv("CASIMIR_NO_GRAPHS") != nullptr;
-    if (no_graphs) {
-        CUDA_TRY(cudaEventRecord(c->ev0, c->stream));
-        launch_steps(c, k);
-        CUDA_TRY(cudaGetLastError());
-        CUDA_TRY(cudaEventRecord(c->ev1, c->stream));
-    }
     auto it = c->graphs.find(k);
-    if (!no_graphs && it == c->graphs.end()) {
+    if (it == c->graphs.end()) {
         std::lock_guard<std::mutex> cg(c->capture_mu);
         cudaGraph_t g;
         CUDA_TRY(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-        launch_steps(c, k);
+        launch_steps(c, k, 0);
         cudaError_t e = cudaStreamEndCapture(c->stream, &g);
         if (e != cudaSuccess) return fail(CASIMIR_ECUDA, std::string("graph capture: ") + cudaGetErrorString(e));
         cudaGraphExec_t ex;
@@ -1315,17 +1372,70 @@ static int run_chunk(casimir_ctx *c, int k)
         if (e != cudaSuccess) return fail(CASIMIR_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
         it = c->graphs.emplace(k, ex).first;
     }
-    if (!no_graphs) {
-        CUDA_TRY(cudaEventRecord(c->ev0, c->stream));
-        CUDA_TRY(cudaGraphLaunch(it->second, c->stream));
-        CUDA_TRY(cudaEventRecord(c->ev1, c->stream));
+    *out = it->second;
+    return CASIMIR_OK;
+}
+
+// Whether every active run is on the resident march.
+static bool only_resident(const casimir_ctx *c)
+{
+    for (const auto &G : c->groups)
+        if (G.ntiles > 0) return false;
+    return c->nres > 0;
+}
+
+// Launch `k` consecutive launch indices.  Resident groups run up to RES_LAUNCH_INDICES of them per launch,
+// beside the step kernels on the last auxiliary streams; the step kernels run as replays of a graph of
+// GRAPH_INDICES indices (and of one index for the rest), or directly when the environment sets
+// CASIMIR_NO_GRAPHS, e.g. for kernel profiling.  (A graph is captured for every set of active runs: one of
+// 64 indices took 16 ms for the Bloch grating's units, of which a 480-step run needs only 13 ms on the device.)
+constexpr int GRAPH_INDICES = 8;
+static int run_chunk(casimir_ctx *c, int k)
+{
+    NvtxRange nvtx_("casimir.chunk");
+    static const bool no_graphs = std::getenv("CASIMIR_NO_GRAPHS") != nullptr;
+    const bool steps = !only_resident(c);
+    if (steps && !no_graphs) {   // captured before anything is launched: the streams take part in the capture
+        cudaGraphExec_t ex;
+        int rc = k >= GRAPH_INDICES ? graph_of(c, GRAPH_INDICES, &ex) : CASIMIR_OK;
+        if (!rc && k % GRAPH_INDICES) rc = graph_of(c, 1, &ex);
+        if (rc) return rc;
     }
+    CUDA_TRY(cudaEventRecord(c->ev0, c->stream));
+    const int nra = steps || c->nres > 1 ? std::min(c->nres, casimir_ctx::NAUX / 2) : 0;   // streams of the resident groups
+    if (nra > 0) CUDA_TRY(cudaEventRecord(c->ev_fork, c->stream));
+    for (int q = 0; q < nra; ++q) CUDA_TRY(cudaStreamWaitEvent(c->aux[casimir_ctx::NAUX - 1 - q], c->ev_fork, 0));
+    for (int q = 0; q < c->nres; ++q) {
+        const auto &G = c->res[q];
+        cudaStream_t st = nra > 0 ? c->aux[casimir_ctx::NAUX - 1 - q % nra] : c->stream;
+        for (int j = 0; j < k; j += RES_LAUNCH_INDICES)
+            launch_res2d(G.shape, (const DevRes2D *)G.sims, G.nsims, c->h_launch + j, std::min(RES_LAUNCH_INDICES, k - j), st);
+    }
+    if (steps && no_graphs) {
+        launch_steps(c, k, nra);
+    } else if (steps) {
+        cudaGraphExec_t ex;
+        int rc = CASIMIR_OK, j = 0;
+        for (; j + GRAPH_INDICES <= k && !rc; j += GRAPH_INDICES)
+            if (!(rc = graph_of(c, GRAPH_INDICES, &ex))) CUDA_TRY(cudaGraphLaunch(ex, c->stream));
+        for (; j < k && !rc; ++j)
+            if (!(rc = graph_of(c, 1, &ex))) CUDA_TRY(cudaGraphLaunch(ex, c->stream));
+        if (rc) return rc;
+    }
+    CUDA_TRY(cudaGetLastError());
+    for (int q = 0; q < nra; ++q) {
+        const int a = casimir_ctx::NAUX - 1 - q;
+        CUDA_TRY(cudaEventRecord(c->ev_join[a], c->aux[a]));
+        CUDA_TRY(cudaStreamWaitEvent(c->stream, c->ev_join[a], 0));
+    }
+    CUDA_TRY(cudaEventRecord(c->ev1, c->stream));
     c->h_launch += k;
     int per_step = 0;
     for (int gi = 0; gi < casimir_ctx::NGROUPS; ++gi)
         if (c->groups[gi].ntiles > 0)
             per_step += ((gi >= 2 && gi < 10) || (gi >= casimir_ctx::G_LINE3 && gi < casimir_ctx::G_CYL)) ? 2 : 1;
-    for (casimir_request *r : c->active) r->launches += (int64_t)k * per_step + c->nres + 1;
+    const int64_t res_launches = (int64_t)c->nres * ((k + RES_LAUNCH_INDICES - 1) / RES_LAUNCH_INDICES);
+    for (casimir_request *r : c->active) r->launches += (int64_t)k * per_step + res_launches + (steps ? (k + GRAPH_INDICES - 1) / GRAPH_INDICES : 0);
     return CASIMIR_OK;
 }
 
@@ -1361,14 +1471,6 @@ static void finish_request(casimir_ctx *c, casimir_request *r, int status)
     r->state.store(status == CASIMIR_OK ? 2 : 3, std::memory_order_release);
 }
 
-// Whether every active run is on the resident march.
-static bool only_resident(const casimir_ctx *c)
-{
-    for (const auto &G : c->groups)
-        if (G.ntiles > 0) return false;
-    return c->nres > 0;
-}
-
 // One engine iteration: run a chunk, then issue copy-backs for finished requests
 // and retire those whose copies landed.  Returns 0 or an error code.
 static int engine_iterate(casimir_ctx *c)
@@ -1387,14 +1489,18 @@ static int engine_iterate(casimir_ctx *c)
         }
         if (rem > 0) {
             int k = (int)std::min<int64_t>(64, rem);
-            const double wd = c->watchdog_ms.load();
-            if (wd > 0 && only_resident(c)) {
-                // the watchdog is checked between chunks: a resident chunk is one launch of up to 192 steps over
-                // every simulation, so it is cut to about a thousandth of the limit (a power of two indices)
-                int cut = 8;
-                if (c->index_ms > 0)
-                    for (cut = 1; cut < 64 && 2 * cut * c->index_ms <= 1e-3 * wd;) cut *= 2;
-                k = std::min(k, cut);
+            if (only_resident(c)) {
+                // short launches go several to a chunk (about 2 ms, between which the host looks at the queue)
+                if (c->index_ms > 0) k = (int)std::min<int64_t>(rem, std::max(64.0, std::min(1024.0, 2.0 / c->index_ms)));
+                // the watchdog is checked between chunks: these are cut to about a thousandth of its limit (a
+                // power of two indices)
+                const double wd = c->watchdog_ms.load();
+                if (wd > 0) {
+                    int cut = 8;
+                    if (c->index_ms > 0)
+                        for (cut = 1; cut < k && 2 * cut * c->index_ms <= 1e-3 * wd;) cut *= 2;
+                    k = std::min(k, cut);
+                }
             }
             int rc = run_chunk(c, k);
             if (rc) return rc;
@@ -1404,7 +1510,8 @@ static int engine_iterate(casimir_ctx *c)
             c->index_ms = ms / k;
             std::lock_guard<std::mutex> lk(c->mu);   // the statistics are read under the lock
             c->step_ms += ms;
-            c->step_launches += only_resident(c) ? c->nres : k;   // one per index, or per chunk where every run is resident
+            // one per index, or per launch where every run is resident
+            c->step_launches += only_resident(c) ? (int64_t)c->nres * ((k + RES_LAUNCH_INDICES - 1) / RES_LAUNCH_INDICES) : k;
             for (auto &aw : c->active_waves) {
                 const casimir_request::Wave &w = aw.first->waves[aw.second];
                 const casimir_plan_t *P = aw.first->plan;
@@ -1582,6 +1689,8 @@ void casimir_ctx_destroy(casimir_ctx_t *c)
         dev_free(c, G.tiles);
     }
     for (auto &G : c->res) dev_free(c, G.sims);
+    for (auto &sp : c->pinned)
+        if (sp.first) cudaFreeHost(sp.first);
     cudaFree(c->d_launch);
     cudaEventDestroy(c->ev0);
     cudaEventDestroy(c->ev1);
@@ -2022,7 +2131,7 @@ int casimir_submit(casimir_plan_t *P, uint64_t tag, casimir_ticket *out)
 
 static void release(casimir_request *r)
 {
-    if (r->h_acc) cudaFreeHost(r->h_acc);
+    give_pinned(r->plan->ctx, r);
     if (r->done_ev) cudaEventDestroy(r->done_ev);
     delete r;
 }
@@ -2108,7 +2217,7 @@ int casimir_run(casimir_plan_t *P, double F[3], double *per_sim, casimir_stats *
             st->kernel_launches = r.launches;
         }
     }
-    if (r.h_acc) cudaFreeHost(r.h_acc);
+    give_pinned(c, &r);
     if (r.done_ev) cudaEventDestroy(r.done_ev);
     if (status != CASIMIR_OK && rc == CASIMIR_OK) return fail(status, "run stopped");
     return status;

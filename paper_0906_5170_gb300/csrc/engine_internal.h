@@ -96,6 +96,7 @@ struct DevPlan {           // device copies of a plan's static tables (kept whil
     DevResWarp *resw = nullptr;
     DevResCta *resc = nullptr;
     DevEntR *rese = nullptr;
+    short *rest = nullptr;
     double *lor = nullptr;
     void *lorc = nullptr;
     void *pml = nullptr;
@@ -129,6 +130,8 @@ struct casimir_plan {
     std::vector<DevResWarp> resW;     // per simulation, [cluster rank][warp]
     std::vector<DevResCta> resC;      // per simulation, [cluster rank]
     std::vector<DevEntR> resE;
+    std::vector<short> resT;          // per simulation, RES_TILES + 1: first piece of each tile
+    std::vector<int> resNT;           // per simulation: tiles
     std::vector<HostTile6> tiles6;
     std::vector<HostTile> tilesM;     // march kernel strip tiles (MARCH_W x MARCH_H) with their entries
     std::vector<DevEnt> entsM;
@@ -162,7 +165,8 @@ struct casimir_request {
     int64_t launches = 0;
     void *block = nullptr;   // fields, acc, tail
     double *acc = nullptr, *tail = nullptr;
-    double *h_acc = nullptr;  // pinned copy-back (acc then tail)
+    double *h_acc = nullptr;  // pinned copy-back (acc, tail, then the status word)
+    size_t h_bytes = 0;
     cudaEvent_t done_ev = nullptr;
     bool copy_issued = false;
     std::vector<double> per_sim;
@@ -222,6 +226,11 @@ struct casimir_ctx {
     };
     std::vector<ResGroup> res;
     int nres = 0;                     // groups in use
+    // pinned result buffers of finished requests, for the next ones (up to PINNED_MAX bytes each)
+    static constexpr int NPINNED = 8;
+    static constexpr size_t PINNED_MAX = 1 << 20;
+    std::pair<double *, size_t> pinned[NPINNED] = {};
+    std::mutex pinned_mu;
     double index_ms = 0;              // time of a launch index in the last chunk
     // waves: simulations are activated in groups whose field bytes fit `wave_bytes`
     // (0: a whole request at once), so that the active working set can stay in L2

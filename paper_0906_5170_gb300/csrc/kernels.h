@@ -200,9 +200,13 @@ struct DevResWarp {        // the rows a warp stages for the surface functional 
     int stage0, stride;    // 16-byte words: the warp's first, and per staging lane
     int gen, pad;          // -1: all its cells are of one material; else its place among those that are not
 };
-struct DevResCta {         // the functional's entries of one CTA, one per thread, by partial sum
-    int e0, ne;
-    short slot[34];        // first entry of partial sum q, q = 0 .. 32
+constexpr int RES_PIECES = 8;   // pieces of a CTA at most
+constexpr int RES_TILES = 16;   // tiles of a functional at most
+struct DevResCta {         // the functional's entries of one CTA, one per thread, by piece (tile of the
+    int e0, ne;            // multi-step kernels) and partial sum
+    short np, rounded;     // pieces; 1: products are rounded before they are added
+    short piece[RES_PIECES];             // their numbers in the simulation (by tile, then CTA)
+    short slot[RES_PIECES * 32 + 1 + 1]; // first entry of each piece's partial sums 0 .. 31
 };
 struct DevEntR {
     int off;               // element within the CTA's staged rows
@@ -215,27 +219,32 @@ struct DevRes2D {
     const DevResCta *ctas;     // [cluster rank]
     const DevEntR *ents;
     int *status;               // set when a wait ran out
-    int64_t carry_off;         // the CTAs' sums between launches, in 16-byte pairs from s.fields
+    const short *tile_pieces;  // [ntile + 1] pieces of each tile
+    int64_t term_off;          // the launch's terms by piece and step, in doubles from s.fields
     int tcols, nb, k;          // threads per row band, row bands, time steps per launch index
     int gen_words;             // 16-byte words of coefficients behind the slots
     int stage_words;           // and of one buffer of staged rows behind them (then the launch's weights)
     int ne_max;                // entries of a CTA at most
-    int shift, pad;            // grid row of the cluster's first row (the grid is a torus)
+    int shift;                 // grid row of the cluster's first row (the grid is a torus)
+    int np_max, ntile_max, ntile;   // pieces of a CTA at most, tiles (of any simulation, and of this one)
 };
 struct Res2dShape {
     int fp64, rb;          // rows of a thread's block
     int cluster, threads, smem;
     int tcols, nb;
     int gen_words, stage_words, ne_max, shift;
+    int np_max, npiece_max, ntile_max;
 };
 int res2d_words(int fp64, int rb, int *coef);   // 16-byte words of a thread's slots, and of its coefficients
 constexpr int RES_CLUSTER_MAX = 16;
 constexpr int RES_SMEM_MAX = 226 * 1024;      // dynamic shared memory of a CTA (the rest is static)
 constexpr int RES_LAUNCH_STEPS = 192;         // time steps of one launch at most (its weights sit in shared memory)
+constexpr int RES_LAUNCH_INDICES = RES_LAUNCH_STEPS / 3;
 cudaError_t res2d_prepare();
-int res2d_proj_bytes(int fp64, int ne);      // shared memory of the projection's history and sums, ne entries a CTA
+int res2d_proj_bytes(const Res2dShape &q);      // shared memory of the projection's history and sums
 std::vector<Res2dShape> res2d_shapes(int fp64, int nx, int ny, int nsims);
-void launch_res2d(const Res2dShape &q, const DevRes2D *sims, int nsims, const int64_t *launch_base, int64_t launch_add, int count, cudaStream_t st);
+// launch indices launch .. launch + count - 1
+void launch_res2d(const Res2dShape &q, const DevRes2D *sims, int nsims, int64_t launch, int count, cudaStream_t st);
 
 void launch_step2d(int fp64, const DevSim2D *sims, const DevTile *tiles, int ntiles,
                    const int64_t *launch_base, int64_t launch_add, cudaStream_t st);

@@ -67,10 +67,6 @@ __device__ __forceinline__ unsigned map_rank(unsigned a, unsigned r)
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(o) : "r"(a), "r"(r));
     return o;
 }
-__device__ __forceinline__ void st_cluster(unsigned a, double v)
-{
-    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
-}
 // 16 bytes to another CTA of the cluster, counted on that CTA's mbarrier when they have landed
 __device__ __forceinline__ void st_async(unsigned a, unsigned mb, const Vec16<float> &v)
 {
@@ -125,6 +121,16 @@ __device__ __forceinline__ bool mb_wait(unsigned mb, unsigned parity)
 template <typename R>
 constexpr bool RES_RED = sizeof(R) == 4;
 
+// (double)v; a float's without the FP64 pipe, which takes 64 clocks for a warp's conversions
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v)
+{
+    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u || m == 0u)   // normal, or zero
+        return __hiloint2double((int)((b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), (int)(b << 29));
+    return (double)v;
+}
+
 // 16-byte words of a thread's slots in shared memory, filled by its neighbours: a row from above (RED: u,
 // else vx), u of the row below, a column from the left (RED: u, else vy), u of the column to the right;
 // RED: two buffers by step parity.  And of the coefficients of its cells, in warps whose cells are not all
@@ -151,23 +157,22 @@ constexpr int F_CU = 24, F_CD = 28;      // CTAs of the bands above and below
 
 template <typename R, int RB, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1)
-k_res2d(const DevRes2D *__restrict__ sims, const int64_t *__restrict__ launch_base, int64_t launch_add, int count)
+k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
 {
     using V4 = Vec16<R>;
     using SL = Slots<R, RB>;
     constexpr int CX = SL::CX, KV = SL::KV;
     constexpr bool RED = RES_RED<R>;
     extern __shared__ __align__(16) unsigned char dyn[];
-    __shared__ double part[2][16];                        // rank 0: the CTAs' sums
-    __shared__ short slot[33];                            // entries of the 32 partial sums
-    __shared__ double tot[2];                             // this CTA's sums over the steps: all, and the tail's
+    __shared__ short slot[RES_PIECES * 32 + 1];           // entries of each piece's 32 partial sums
+    __shared__ short piece[RES_PIECES];                   // the simulation's numbers of this CTA's pieces
     __shared__ __align__(8) unsigned long long mbar[4];   // rows from the previous and from the next CTA, by step parity
 
     const unsigned C = cluster_size(), rank = cluster_rank();
     const DevRes2D &D = sims[blockIdx.x / C];
     const DevSim2D &S = D.s;
     // the launch indices of this launch and the time steps they hold (the same for the whole cluster)
-    const int64_t L0 = *launch_base + launch_add - S.s0;
+    const int64_t L0 = launch - S.s0;
     const int64_t l_lo = L0 > 1 ? L0 : 1, l_hi = L0 + count - 1;
     if (l_hi < l_lo || (l_lo - 1) * D.k + 1 > S.T) return;
     const int n_lo = (int)((l_lo - 1) * D.k + 1), n_hi = (int)min((int64_t)S.T, l_hi * D.k);
@@ -229,13 +234,19 @@ k_res2d(const DevRes2D *__restrict__ sims, const int64_t *__restrict__ launch_ba
     // of RES_WIN steps, and every RES_WIN steps the CTA forms s(n) = sum_e w_e F_e(n) of the window's steps,
     // one lane per step and group of entries (in FP64; GB300's FP64 pipe takes 64 clocks per warp
     // instruction, which a reduction per step put on the critical path of every step).
-    // The sums go over one step after the other, however the steps are cut into launches.
+    // The terms w_n s(n) go to the second field buffer (unused otherwise), and rank 0 adds them at the end of the launch as the multi-step kernels do: by
+    // tile and launch index (a CTA's entries of one tile are a piece).  The sum over a run's steps is rounded
+    // to the last bit of its early terms thousands of times, the force is a small difference of such sums, and
+    // in this order they round as before and do not depend on how the steps were cut into launches.
     const DevResWarp pw = D.warps[(int)rank * (nt >> 5) + warp];
     unsigned pk_stage;             // first staged word (16 bits), element of this thread's entry (16 bits)
     const int stage_w = nt * SL::WORDS + D.gen_words, sbuf = D.stage_words, nem = D.ne_max;
-    // behind the staged rows: this launch's weights, the entries' weights, partial sums, the history
+    const int np = D.ctas[rank].np, rounded = D.ctas[rank].rounded;
+    // behind the staged rows: this launch's weights, the entries' weights, partial sums, ..., the history
+    const int n_tail = S.tail_from + 1;                            // the first step of the tail's sums
     const int gw_i = (stage_w + 2 * sbuf) * 2, we_i = gw_i + RES_LAUNCH_STEPS, ps_i = we_i + nem;
-    const int hist_i = (ps_i + 16 * RES_WIN) * (int)(8 / sizeof(R));
+    const int at_i = ps_i + D.np_max * 16 * RES_WIN;   // rank 0: the terms by tile and launch index
+    const int hist_i = (at_i + 2 * D.ntile_max * RES_LAUNCH_INDICES) * (int)(8 / sizeof(R));
     double *const dd = reinterpret_cast<double *>(dyn);
     {
         flags |= ((pw.lanes >> lane) & 1) ? F_STAGE : 0u;
@@ -245,18 +256,14 @@ k_res2d(const DevRes2D *__restrict__ sims, const int64_t *__restrict__ launch_ba
         for (int i = t; i < cnt; i += nt) dd[gw_i + i] = S.gw[n_lo - 1 + i];
         const DevResCta &pc = D.ctas[rank];
         int off = 0;
-        for (int q = t; q < 33; q += nt) slot[q] = pc.slot[q];
+        for (int q = t; q < RES_PIECES * 32 + 1; q += nt) slot[q] = pc.slot[q];
+        if (t < RES_PIECES) piece[t] = pc.piece[t];
         if (t < pc.ne) {
             flags |= F_MINE;
             off = D.ents[pc.e0 + t].off;
             dd[we_i + t] = D.ents[pc.e0 + t].w;
         }
         pk_stage = (unsigned)st | (unsigned)off << 16;
-        if (t == 0) {
-            const double2 v = (reinterpret_cast<const double2 *>(S.fields) + D.carry_off)[rank];
-            tot[0] = v.x;
-            tot[1] = v.y;
-        }
     }
 
     // the fields of the block with vx of the row above (vxm) and vy of the column to the left (vym), which
@@ -353,52 +360,58 @@ k_res2d(const DevRes2D *__restrict__ sims, const int64_t *__restrict__ launch_ba
             if ((flags & lead) && i + 2 < cnt) mb_expect(m, D.tcols * 16);
         }
     };
-    // Sums of the steps of window k that lie in [n_lo, last], in the order of the other 2D kernels: 32 partial
-    // sums (an entry's is its place in its row) of rounded products, added as a warp's shuffles add its lanes.
-    auto flush = [&](int k, int last) {
+    // Sums of the steps of window k that lie in [n_lo, last]: 32 partial sums a piece, added as a warp's shuffles
+    // add its lanes (on horizontal faces an entry's partial sum is its place in its row and the products are
+    // rounded, as in the other 2D kernels).  A half warp takes one partial sum, a lane of it one step; with
+    // entries in the first 16 alone, the halves take neighbouring ones.
+    auto part_sums = [&](int k, int last) {
         const int ln = (int)threadIdx.x & 31, half = ln / RES_WIN, st = ln & (RES_WIN - 1), n = k * RES_WIN + st;
-        const bool in = n >= n_lo && n <= last;
-        if (in) {
-            const R *const hs = reinterpret_cast<const R *>(dyn) + hist_i + (n & (2 * RES_WIN - 1)) * nem;
-            for (int g = 2 * ((int)threadIdx.x >> 5) + half; g < 16; g += (int)blockDim.x >> 4) {
-                double p = 0.0, q = 0.0;
-                for (int e = slot[g]; e < slot[g + 1]; ++e) p = __dadd_rn(p, __dmul_rn(dd[we_i + e], (double)hs[e]));
-                for (int e = slot[g + 16]; e < slot[g + 17]; ++e) q = __dadd_rn(q, __dmul_rn(dd[we_i + e], (double)hs[e]));
-                dd[ps_i + g * RES_WIN + st] = p + q;
-            }
-        }
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            double s = 0.0;
-            if (in) {
-                const double *const ps = dd + ps_i + half * RES_WIN + st;   // groups half, half + 2, ...
-                const double a0 = ps[0] + ps[8 * RES_WIN], a2 = ps[2 * RES_WIN] + ps[10 * RES_WIN];
-                const double a4 = ps[4 * RES_WIN] + ps[12 * RES_WIN], a6 = ps[6 * RES_WIN] + ps[14 * RES_WIN];
-                s = (a0 + a4) + (a2 + a6);
-            }
-            s += __shfl_down_sync(0xffffffffu, s, RES_WIN);
-            if (half == 0) dd[ps_i + st] = in ? dd[gw_i + n - n_lo] * s : 0.0;   // (this lane alone reads and writes column st)
-            __syncwarp();
-            if (threadIdx.x == 0) {   // one step after the other: consecutive terms cancel
-                double acc = tot[0], tail = tot[1];
-                for (int v = max(n_lo, k * RES_WIN); v <= last; ++v) {
-                    const double c = dd[ps_i + v - k * RES_WIN];
-                    acc += c;
-                    if (v > S.tail_from) tail += c;
+        const R *const hs = reinterpret_cast<const R *>(dyn) + hist_i + (n & (2 * RES_WIN - 1)) * nem;
+        for (int pc = 0; pc < np; ++pc) {
+            const short *const sl = slot + 32 * pc;
+            const bool low = sl[16] == sl[32];
+            for (int q = (int)threadIdx.x >> 5; q < (low ? 8 : 16); q += (int)blockDim.x >> 5) {
+                double p = 0.0;
+                const int g = low ? 2 * q + half : q + 16 * half;
+                int e = sl[g];
+                const int e1 = sl[g + 1];
+                if (e < e1 && n >= n_lo && n <= last) {
+                    p = dd[we_i + e] * widen(hs[e]);
+                    if (rounded)
+                        for (++e; e < e1; ++e) p = __dadd_rn(p, __dmul_rn(dd[we_i + e], widen(hs[e])));
+                    else
+                        for (++e; e < e1; ++e) p = fma(dd[we_i + e], widen(hs[e]), p);
                 }
-                tot[0] = acc;
-                tot[1] = tail;
+                if (!low) p += __shfl_down_sync(0xffffffffu, p, RES_WIN);
+                if (low || half == 0) dd[ps_i + (pc * 16 + (g & 15)) * RES_WIN + st] = p;
             }
         }
     };
+    auto add_window = [&](int k, int last) {   // by the last warps, after the barrier that follows part_sums
+        const int nw = (int)blockDim.x >> 5;
+        for (int pc = nw - 1 - ((int)threadIdx.x >> 5); pc < np; pc += nw) {
+            const int ln = (int)threadIdx.x & 31, half = ln / RES_WIN, st = ln & (RES_WIN - 1), n = k * RES_WIN + st;
+            const double *const ps = dd + ps_i + (pc * 16 + half) * RES_WIN + st;   // groups half, half + 2, ...
+            const double a0 = ps[0] + ps[8 * RES_WIN], a2 = ps[2 * RES_WIN] + ps[10 * RES_WIN];
+            const double a4 = ps[4 * RES_WIN] + ps[12 * RES_WIN], a6 = ps[6 * RES_WIN] + ps[14 * RES_WIN];
+            double s = (a0 + a4) + (a2 + a6);
+            s += __shfl_down_sync(0xffffffffu, s, RES_WIN);
+            if (half == 0 && n >= n_lo && n <= last)
+                reinterpret_cast<double *>(S.fields)[D.term_off + piece[pc] * RES_LAUNCH_STEPS + (n - n_lo)] = dd[gw_i + n - n_lo] * s;
+        }
+    };
     // the entries' values of the launch's step i, staged before the last barrier, join the history; a window
-    // whose last step joined it before that barrier is summed (the same for every warp of the CTA)
+    // whose last step joined it before that barrier is summed, and added a step later (the same for every
+    // warp of the CTA)
     auto consume = [&](int i) {
         const int n = n_lo + i;
         if (flags & F_MINE)
             reinterpret_cast<R *>(dyn)[hist_i + (n & (2 * RES_WIN - 1)) * nem + (int)threadIdx.x] =
                 reinterpret_cast<const R *>(blocks + stage_w + (i & 1) * sbuf)[pk_stage >> 16];
-        if (i > 0 && (n & (RES_WIN - 1)) == 0) flush((n - 1) / RES_WIN, n - 1);
+        if (nem > 0 && (n & (RES_WIN - 2)) == 0) {
+            if ((n & 1) == 0 && i > 0) part_sums((n - 1) / RES_WIN, n - 1);
+            if ((n & 1) == 1 && i > 1) add_window((n - 2) / RES_WIN, n - 2);
+        }
     };
     auto put_row = [&](unsigned far, int at, unsigned cta, unsigned mb, const V4 &v) {
         if (flags & far) st_async(map_rank((unsigned)__cvta_generic_to_shared(blocks + at), cta), map_rank(mb, cta), v);
@@ -521,7 +534,32 @@ k_res2d(const DevRes2D *__restrict__ sims, const int64_t *__restrict__ launch_ba
             }
         };
         [[maybe_unused]] constexpr bool HAS_INNER = RB > 3 && CX > 2;   // cells whose u no neighbour needs
-        // V phase: the part no neighbour's u enters, the step's barrier, the rest
+        // RED: vx of the row above from its u
+        auto v_up = [&](const V4 *own) {
+            if constexpr (RED) {
+                const V4 hu = own[SL::UP], k = row(0, -1);
+#pragma unroll
+                for (int c = 0; c < CX; ++c) vxm[RED ? c : 0] = upx(vxm[RED ? c : 0], k.c[c], u[0][c] - hu.c[c]);
+            }
+        };
+        // vx of the last rows from u of the row below
+        auto v_down = [&](const V4 *own) {
+            const V4 hd = own[SL::DN];
+            if (RB > 1) {
+                // a band of RB - 1 rows keeps its neighbour's row 0 in its last row
+                const bool cut = flags & F_SHORT;
+#pragma unroll
+                for (int c = 0; c < CX; ++c) u[RB - 1][c] = cut ? hd.c[c] : u[RB - 1][c];
+                const V4 k = row(0, RB > 1 ? RB - 2 : 0);
+#pragma unroll
+                for (int c = 0; c < CX; ++c)
+                    vx[RB > 1 ? RB - 2 : 0][c] = upx(vx[RB > 1 ? RB - 2 : 0][c], k.c[c], u[RB - 1][c] - u[RB > 1 ? RB - 2 : 0][c]);
+            }
+            const V4 k = row(0, RB - 1);
+#pragma unroll
+            for (int c = 0; c < CX; ++c) vx[RB - 1][c] = upx(vx[RB - 1][c], k.c[c], hd.c[c] - u[RB - 1][c]);
+        };
+        // V phase: the part no neighbour's u enters, the step's barrier, the columns at the sides (RED), the rest
         auto phase_v = [&](int i) {
             const V4 *const own = blocks + (int)threadIdx.x * SL::WORDS + (RED ? (i & 1) * SL::BUF : 0);
             if (flags & F_LATE) {
@@ -570,28 +608,9 @@ k_res2d(const DevRes2D *__restrict__ sims, const int64_t *__restrict__ launch_ba
                         vy[r][CX - 1] = upy(vy[r][CX - 1], one(1, r, CX - 1), hr.c[c] - u[r][CX - 1]);
                     }
             }
-            if constexpr (RED) {
-                wait_far(F_NEEDU, F_LEADU, mb_u, i);
-                const V4 hu = own[SL::UP], k = row(0, -1);
-#pragma unroll
-                for (int c = 0; c < CX; ++c) vxm[RED ? c : 0] = upx(vxm[RED ? c : 0], k.c[c], u[0][c] - hu.c[c]);
-            }
-            wait_far(F_NEEDD, F_LEADD, mb_d, i);
-            const V4 hd = own[SL::DN];
-            if (RB > 1) {
-                // a band of RB - 1 rows keeps its neighbour's row 0 in its last row
-                const bool cut = flags & F_SHORT;
-#pragma unroll
-                for (int c = 0; c < CX; ++c) u[RB - 1][c] = cut ? hd.c[c] : u[RB - 1][c];
-                const V4 k = row(0, RB > 1 ? RB - 2 : 0);
-#pragma unroll
-                for (int c = 0; c < CX; ++c)
-                    vx[RB > 1 ? RB - 2 : 0][c] = upx(vx[RB > 1 ? RB - 2 : 0][c], k.c[c], u[RB - 1][c] - u[RB > 1 ? RB - 2 : 0][c]);
-            }
-            {
-                const V4 k = row(0, RB - 1);
-#pragma unroll
-                for (int c = 0; c < CX; ++c) vx[RB - 1][c] = upx(vx[RB - 1][c], k.c[c], hd.c[c] - u[RB - 1][c]);
+            if constexpr (!RED) {
+                wait_far(F_NEEDD, F_LEADD, mb_d, i);
+                v_down(own);
             }
         };
         // U phase without RED: the part no neighbour's v enters, the barrier, the rest
@@ -658,6 +677,11 @@ k_res2d(const DevRes2D *__restrict__ sims, const int64_t *__restrict__ launch_ba
             asm volatile("" : "+r"(flags), "+r"(pk_row), "+r"(pk_col), "+r"(pk_stage));
             if constexpr (RED) {
                 phase_v(i);
+                const V4 *const own = blocks + (int)threadIdx.x * SL::WORDS + (i & 1) * SL::BUF;
+                wait_far(F_NEEDU, F_LEADU, mb_u, i);
+                v_up(own);
+                wait_far(F_NEEDD, F_LEADD, mb_d, i);
+                v_down(own);
                 if (!SU) stage(i);
                 if (SU || i + 1 < cnt) {
 #pragma unroll
@@ -727,33 +751,48 @@ k_res2d(const DevRes2D *__restrict__ sims, const int64_t *__restrict__ launch_ba
                     }
         }
     }
-    // the last window: consume() sums one when the first step of the next has joined the history
+    // the last window, and the one before it when its partial sums are the last thing consume() did
     __syncthreads();
-    flush(n_hi / RES_WIN, n_hi);
-    // the sums so far, added in the order of the CTAs
-    const unsigned rk = cluster_rank(), cs = cluster_size();
-    if (t2 == 0) {
-        (reinterpret_cast<double2 *>(S.fields) + D.carry_off)[rk] = make_double2(tot[0], tot[1]);
-        if (cs > 1) {
-            st_cluster(map_rank((unsigned)__cvta_generic_to_shared(&part[0][rk]), 0), tot[0]);
-            st_cluster(map_rank((unsigned)__cvta_generic_to_shared(&part[1][rk]), 0), tot[1]);
-        } else {
-            part[0][0] = tot[0];
-            part[1][0] = tot[1];
-        }
-    }
+    if (cnt > 1 && (n_hi & (RES_WIN - 1)) == 0) add_window((n_hi - 1) / RES_WIN, n_hi - 1);
+    __syncthreads();
+    part_sums(n_hi / RES_WIN, n_hi);
+    __syncthreads();
+    add_window(n_hi / RES_WIN, n_hi);
     if (dead) *D.status = 1;
-    if (cs > 1) {
+    // rank 0 adds the terms to the simulation's sums
+    const unsigned rk = cluster_rank();
+    if (cluster_size() > 1) {
         __syncwarp();
         cluster_sync();
+    } else {
+        __syncthreads();
     }
-    if (rk == 0 && t2 == 0) {
-        double acc = 0.0, tail = 0.0;
-        for (unsigned v = 0; v < cs; ++v) {
-            acc += part[0][v];
-            tail += part[1][v];
+    if (rk != 0) return;
+    const int K = D.k, nt_ = D.ntile, total = (cnt + K - 1) / K * nt_;
+    const short *const tp = D.tile_pieces;
+    for (int x = t2; x < total; x += (int)blockDim.x) {
+        const int l = x / nt_, tl = x - l * nt_;
+        double c = 0.0, ct = 0.0;
+        for (int i = l * K; i < min(cnt, l * K + K); ++i) {
+            double cq = 0.0;
+            for (int p = tp[tl]; p < tp[tl + 1]; ++p) cq += reinterpret_cast<volatile const double *>(S.fields)[D.term_off + p * RES_LAUNCH_STEPS + i];
+            c += cq;
+            if (n_lo + i >= n_tail) ct += cq;
         }
+        dd[at_i + x] = c;
+        dd[at_i + D.ntile_max * RES_LAUNCH_INDICES + x] = ct;
+    }
+    __syncthreads();
+    if (t2 == 0) {
+        double acc = *S.acc;
+#pragma unroll 8
+        for (int x = 0; x < total; ++x) acc += dd[at_i + x];
         *S.acc = acc;
+    }
+    if (t2 == (int)blockDim.x - 1 && n_hi >= n_tail) {
+        double tail = *S.tail;
+#pragma unroll 8
+        for (int x = 0; x < total; ++x) tail += dd[at_i + D.ntile_max * RES_LAUNCH_INDICES + x];
         *S.tail = tail;
     }
 }
@@ -779,7 +818,12 @@ int res2d_words(int fp64, int rb, int *coef)   // Slots<R, rb>::WORDS, CWORDS
     return ((1 + red) * (2 + 2 * kv)) | 1;
 }
 
-int res2d_proj_bytes(int fp64, int ne) { return (ne + 16 * RES_WIN) * 8 + 2 * RES_WIN * ne * (fp64 ? 8 : 4); }
+int res2d_proj_bytes(const Res2dShape &q)
+{
+    const int rs = q.fp64 ? 8 : 4;
+    return (q.ne_max + q.np_max * 16 * RES_WIN + 2 * q.ntile_max * RES_LAUNCH_INDICES) * 8 +
+           (2 * RES_WIN * q.ne_max * rs + 15) / 16 * 16;
+}
 
 cudaError_t res2d_prepare()
 {
@@ -811,14 +855,14 @@ static cudaError_t launch_cfg(const void *k, int grid, int cluster, int threads,
     return k ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-void launch_res2d(const Res2dShape &q, const DevRes2D *sims, int nsims, const int64_t *launch_base, int64_t launch_add, int count, cudaStream_t st)
+void launch_res2d(const Res2dShape &q, const DevRes2D *sims, int nsims, int64_t launch, int count, cudaStream_t st)
 {
     if (nsims <= 0) return;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at;
     const void *k = res2d_kernel(q.fp64, q.rb);
     if (launch_cfg(k, nsims * q.cluster, q.cluster, q.threads, q.smem, st, &cfg, &at) != cudaSuccess) return;
-    void *args[] = {(void *)&sims, (void *)&launch_base, (void *)&launch_add, (void *)&count};
+    void *args[] = {(void *)&sims, (void *)&launch, (void *)&count};
     cudaLaunchKernelExC(&cfg, k, args);
 }
 
