@@ -95,7 +95,8 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
     P->resT.clear();
     P->resNT.clear();
     q->stage_words = q->ne_max = q->np_max = q->npiece_max = q->ntile_max = 0;
-    const int txk = tile_xk(P->opts.steps_per_launch == 3 ? 3 : 2), tx = (nx + txk - 1) / txk;   // tiles of the multi-step kernels
+    const int txk = q->cyl ? MARCH_W2 : tile_xk(P->opts.steps_per_launch == 3 ? 3 : 2), tx = (nx + txk - 1) / txk;   // tiles of the multi-step kernels
+    const int tyk = q->cyl ? P->opts.march_rows : TILE_Y;
     // the cluster's first row: the first that leaves the rows of every horizontal face in one CTA
     std::map<int, std::pair<int, int>> span;   // face -> its measured rows
     for (const Sim &sm : D.sims)
@@ -122,9 +123,9 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
     }
     // warps whose cells (FP32: with the row above and the column to the left of each thread's block) hold more
     // than one material keep their coefficients in shared memory (per geometry)
-    const int halo = q->fp64 ? 0 : 1;
+    const int halo = q->fp64 || q->cyl ? 0 : 1;
     int cwords = 0, gen_max = 0;
-    res2d_words(q->fp64, q->rb, &cwords);
+    res_words(q->cyl, q->fp64, q->rb, &cwords);
     std::map<int, std::vector<int>> gen;
     auto gen_of = [&](int geo) -> const std::vector<int> & {
         auto it = gen.find(geo);
@@ -158,7 +159,13 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
     std::vector<DevResWarp> rec((size_t)q->cluster * nwarp);
     for (const Sim &sm : D.sims) {
         std::fill(rec.begin(), rec.end(), DevResWarp{});
-        const int arrays = sm.second_u ? 1 : 2;
+        const int arrays = q->cyl ? 3 : (sm.second_u ? 1 : 2);
+        // the sigma group's first array; cylindrical: the entries of the source's real set alone (prepare_plan)
+        const int arr0 = q->cyl ? 3 * sm.kind : (sm.second_u ? 0 : 1);
+        auto in_a = [](int arr) { return arr == 0 || arr == 1 || arr == 5; };
+        std::vector<Entry> meas;
+        for (const Entry &e : sm.meas)
+            if (!q->cyl || sm.src.empty() || in_a(e.arr) == in_a(sm.src[0].arr)) meas.push_back(e);
         // the place of an entry: CTA, warp record, lane, row and element of the block
         auto place = [&](const Entry &e, int *cta, int *lane, int *row, int *el) -> DevResWarp & {
             const int i = (int)(e.idx % nx), j = (int)((e.idx / nx - q->shift + ny) % ny);   // the cluster's row
@@ -171,8 +178,8 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
             return rec[(size_t)r * nwarp + t / 32];
         };
         int cta, lane, row, el;
-        for (const Entry &e : sm.meas) {
-            if (sm.second_u ? e.arr != 0 : (e.arr != 1 && e.arr != 2)) return false;   // the sigma group only
+        for (const Entry &e : meas) {
+            if (e.arr < arr0 || e.arr >= arr0 + arrays) return false;   // the sigma group only
             DevResWarp &w = place(e, &cta, &lane, &row, &el);
             w.lanes |= 1u << lane;
             w.rows |= 1u << row;
@@ -192,7 +199,7 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
         // on a horizontal face an entry's partial sum is its place in its grid row (modulo 32), as in the tiles of
         // the multi-step kernels; elsewhere the entries are dealt to the first 16 in turn
         std::vector<std::pair<int64_t, const Entry *>> order;
-        for (const Entry &e : sm.meas) order.push_back({e.idx, &e});
+        for (const Entry &e : meas) order.push_back({e.idx, &e});
         std::stable_sort(order.begin(), order.end(), [](const auto &x, const auto &y) { return x.first < y.first; });
         int64_t row_at = -1;
         int place_in_row = 0;
@@ -200,7 +207,7 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
         std::map<std::pair<int, int>, int> pieces;                                   // (tile, CTA) -> number
         for (const auto &oe : order) {
             const Entry &e = *oe.second;
-            const int ti = (int)(e.idx % nx) / txk, tile = (int)(e.idx / nx) / TILE_Y * tx + ti;
+            const int ti = (int)(e.idx % nx) / txk, tile = (int)(e.idx / nx) / tyk * tx + ti;
             const int64_t at = e.idx / nx * tx + ti;   // the row of the tile
             if (at != row_at && D.faces[sm.face].axis == 1) {
                 row_at = at;
@@ -209,7 +216,7 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
             const int sum = place_in_row++ % (D.faces[sm.face].axis == 1 ? 32 : 16);
             const DevResWarp &w = place(e, &cta, &lane, &row, &el);
             const int word = w.stage0 + __builtin_popcount(w.lanes & ((1u << lane) - 1u)) * w.stride +
-                             __builtin_popcount(w.rows & ((1u << row) - 1u)) * arrays + (sm.second_u ? 0 : e.arr - 1);
+                             __builtin_popcount(w.rows & ((1u << row) - 1u)) * arrays + e.arr - arr0;
             byp[cta].push_back({tile, DevEntR{word * cx + el, sum, e.re}});
             pieces[{tile, cta}] = 0;
         }
@@ -258,10 +265,10 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
         }
         P->resW.insert(P->resW.end(), rec.begin(), rec.end());
     }
-    if ((int64_t)q->npiece_max * RES_LAUNCH_STEPS * 8 + 8 > 3 * (int64_t)nx * ny * (int64_t)P->rsize) return false;   // their terms wait in the second field buffer
+    if ((int64_t)q->npiece_max * RES_LAUNCH_STEPS * 8 + 8 > (q->cyl ? 6 : 3) * (int64_t)nx * ny * (int64_t)P->rsize) return false;   // their terms wait in the second field buffer
     q->gen_words = gen_max * 32 * cwords;
-    q->smem += 16 * (q->gen_words + 2 * q->stage_words) + res2d_proj_bytes(*q);
-    if (nwarp * 32 * res2d_words(q->fp64, q->rb, &cwords) + q->gen_words + 2 * q->stage_words >= 1 << 16) return false;   // packed into 16 bits
+    q->smem += 16 * (q->gen_words + 2 * q->stage_words) + res2d_proj_bytes(*q);   // (the radial factors are in smem already)
+    if (nwarp * 32 * res_words(q->cyl, q->fp64, q->rb, &cwords) + q->gen_words + 8 * q->tcols + 2 * q->stage_words >= 1 << 16) return false;   // packed into 16 bits
     return q->smem <= RES_SMEM_MAX;
 }
 
@@ -320,11 +327,12 @@ static int prepare_plan(casimir_plan_t *P, bool allow_resident)
             }
         P->pml_off.push_back(po);
     }
-    // 2D TM/TE plans on a device: the first shape of the resident march that holds them
-    if (allow_resident && P->ctx && !D.sims.empty() && D.geos[D.sims[0].geo].family != FAM_FULL &&
-        6 * (int64_t)D.prob.n[0] * D.prob.n[1] < ((int64_t)1 << 31)) {
+    // 2D TM/TE and cylindrical plans on a device: the first shape of the resident march that holds them
+    const bool cyl = !D.sims.empty() && D.geos[D.sims[0].geo].cyl;
+    if (allow_resident && P->ctx && !D.sims.empty() && (cyl || D.geos[D.sims[0].geo].family != FAM_FULL) &&
+        12 * (int64_t)D.prob.n[0] * D.prob.n[1] < ((int64_t)1 << 31)) {
         cudaSetDevice(P->ctx->device);
-        for (Res2dShape &q : res2d_shapes(P->fp64, D.prob.n[0], D.prob.n[1], (int)D.sims.size()))
+        for (Res2dShape &q : res2d_shapes(cyl, P->fp64, D.prob.n[0], D.prob.n[1], (int)D.sims.size()))
             if (resident_tables(P, &q)) {
                 P->resident = true;
                 P->res = q;
@@ -532,7 +540,12 @@ static int prepare_plan(casimir_plan_t *P, bool allow_resident)
                     for (int q = 0; q < g.npoles; ++q)
                         for (int c = 0; c < 3; ++c)
                             if (g.lorentz[((size_t)id * g.npoles + q) * 6 + 2 * c] != 0.0) geo_poles = std::max(geo_poles, q + 1);
-                if (P->opts.steps_per_launch >= 2 && (hs.cyl || (!P->fp64 && geo_poles <= 1))) {
+                if (P->resident) {
+                    hs.resw0 = (int64_t)s * P->res.cluster * (P->res.threads / 32);
+                    hs.resc0 = (int64_t)s * P->res.cluster;
+                    hs.rese0 = rese;
+                    for (int v = 0; v < P->res.cluster; ++v) rese += P->resC[hs.resc0 + v].ne;
+                } else if (P->opts.steps_per_launch >= 2 && (hs.cyl || (!P->fp64 && geo_poles <= 1))) {
                     // MARCH_W2-wide strips, entries sorted by row with per-row offsets (the sigma
                     // group is projected from registers)
                     const int tx2 = (hs.nx + MARCH_W2 - 1) / MARCH_W2;
@@ -743,7 +756,7 @@ static int prepare_plan(casimir_plan_t *P, bool allow_resident)
         bool all2d = !P->sims.empty() && !P->sims[0].full;
         // six-component runs fuse two steps when every simulation has its two-step tiles
         bool two6 = !P->sims.empty() && !all2d;
-        for (const HostSim &h : P->sims) two6 = two6 && h.march && h.ntile2 > 0;
+        for (const HostSim &h : P->sims) two6 = two6 && h.march && (h.ntile2 > 0 || P->resident);
         P->k2d = all2d ? P->opts.steps_per_launch : (two6 ? 2 : 1);
         P->launches = (D.prob.n_steps + P->k2d - 1) / P->k2d;
     }
@@ -759,7 +772,7 @@ static int prepare_plan(casimir_plan_t *P, bool allow_resident)
     P->request_bytes = (int64_t)(align256(P->field_elems * P->rsize) + 2 * align256((P->sims.size() + 1) * 8) +
                                  P->tiles.size() * sizeof(DevTile) + P->tiles6.size() * sizeof(DevTile6) +
                                  P->tiles2.size() * sizeof(DevTile2) + P->tilesM.size() * sizeof(DevTile) +
-                                 P->sims.size() * std::max(sizeof(DevRes2D), sizeof(DevSim6)));
+                                 P->sims.size() * std::max(sizeof(DevResCyl), sizeof(DevSim6)));
     return CASIMIR_OK;
 }
 
@@ -1080,7 +1093,7 @@ static int rebuild(casimir_ctx *c)
     std::vector<DevTile2> tc2[2];
     std::vector<DevSim6> sm2[2 * MAR2_VARIANTS];    // Cartesian march, two steps per launch
     std::vector<DevTile2> tm2[2 * MAR2_VARIANTS];
-    std::vector<std::pair<Res2dShape, std::vector<DevRes2D>>> res;   // resident 2D runs by shape
+    std::vector<std::pair<Res2dShape, std::vector<char>>> res;   // resident runs' descriptors by shape
     for (auto &aw : c->active_waves) {
         casimir_request *r = aw.first;
         const casimir_request::Wave &w = r->waves[aw.second];
@@ -1091,28 +1104,42 @@ static int rebuild(casimir_ctx *c)
             if (P->resident) {
                 const Res2dShape &q = P->res;
                 size_t gi = 0;
-                while (gi < res.size() && !(res[gi].first.fp64 == q.fp64 && res[gi].first.rb == q.rb && res[gi].first.cluster == q.cluster &&
-                                            res[gi].first.threads == q.threads && res[gi].first.smem == q.smem)) ++gi;
+                while (gi < res.size() && !(res[gi].first.fp64 == q.fp64 && res[gi].first.cyl == q.cyl && res[gi].first.rb == q.rb &&
+                                            res[gi].first.cluster == q.cluster && res[gi].first.threads == q.threads && res[gi].first.smem == q.smem)) ++gi;
                 if (gi == res.size()) res.push_back({q, {}});
-                DevRes2D d{};
-                make_sim2d(P, blk, r->acc, r->tail, w.s0, s, &d.s);
-                d.warps = P->dev.resw + hs.resw0;
-                d.ctas = P->dev.resc + hs.resc0;
-                d.ents = P->dev.rese + hs.rese0;
-                d.status = (int *)(r->tail + P->sims.size());
-                d.gen_words = q.gen_words;
-                d.stage_words = q.stage_words;
-                d.ne_max = q.ne_max;
-                d.shift = q.shift;
-                d.tile_pieces = P->dev.rest + s * (RES_TILES + 1);
-                d.ntile = P->resNT[s];
-                d.np_max = q.np_max;
-                d.term_off = (3 * (int64_t)hs.nx * hs.ny * (int64_t)P->rsize + 7) / 8;   // the second field buffer
-                d.ntile_max = q.ntile_max;
-                d.tcols = q.tcols;
-                d.nb = q.nb;
-                d.k = P->k2d;
-                res[gi].second.push_back(d);
+                auto ext = [&](DevRes &d) {
+                    d.warps = P->dev.resw + hs.resw0;
+                    d.ctas = P->dev.resc + hs.resc0;
+                    d.ents = P->dev.rese + hs.rese0;
+                    d.status = (int *)(r->tail + P->sims.size());
+                    d.gen_words = q.gen_words;
+                    d.stage_words = q.stage_words;
+                    d.ne_max = q.ne_max;
+                    d.shift = q.shift;
+                    d.tile_pieces = P->dev.rest + s * (RES_TILES + 1);
+                    d.ntile = P->resNT[s];
+                    d.np_max = q.np_max;
+                    d.ntile_max = q.ntile_max;
+                    d.term_off = ((q.cyl ? 6 : 3) * (int64_t)hs.nx * hs.ny * (int64_t)P->rsize + 7) / 8;   // the second field buffer
+                    d.tcols = q.tcols;
+                    d.nb = q.nb;
+                    d.k = P->k2d;
+                };
+                auto put = [&](const auto &d) {
+                    const char *p = reinterpret_cast<const char *>(&d);
+                    res[gi].second.insert(res[gi].second.end(), p, p + sizeof(d));
+                };
+                if (q.cyl) {
+                    DevResCyl d{};
+                    make_sim6(P, blk, r->acc, r->tail, w.s0, s, &d.s);
+                    ext(d);
+                    put(d);
+                } else {
+                    DevRes2D d{};
+                    make_sim2d(P, blk, r->acc, r->tail, w.s0, s, &d.s);
+                    ext(d);
+                    put(d);
+                }
             } else if (!hs.full) {
                 auto &sv = s2[P->fp64];
                 auto &tv = t2[P->fp64];
@@ -1269,12 +1296,12 @@ static int rebuild(casimir_ctx *c)
     if (c->res.size() < res.size()) c->res.resize(res.size());
     for (size_t gi = 0; gi < res.size(); ++gi) {
         auto &G = c->res[gi];
-        const size_t bytes = res[gi].second.size() * sizeof(DevRes2D);
+        const size_t bytes = res[gi].second.size();
         int rc = grow(c, &G.sims, &G.cap, bytes);
         if (rc) return rc;
         CUDA_TRY(cudaMemcpyAsync(G.sims, res[gi].second.data(), bytes, cudaMemcpyHostToDevice, c->stream));
         G.shape = res[gi].first;
-        G.nsims = (int)res[gi].second.size();
+        G.nsims = (int)(bytes / (G.shape.cyl ? sizeof(DevResCyl) : sizeof(DevRes2D)));
         c->ntiles += G.nsims;
     }
     // the launch counter of the step kernels (resident runs take the index from the host)
@@ -1409,7 +1436,7 @@ static int run_chunk(casimir_ctx *c, int k)
         const auto &G = c->res[q];
         cudaStream_t st = nra > 0 ? c->aux[casimir_ctx::NAUX - 1 - q % nra] : c->stream;
         for (int j = 0; j < k; j += RES_LAUNCH_INDICES)
-            launch_res2d(G.shape, (const DevRes2D *)G.sims, G.nsims, c->h_launch + j, std::min(RES_LAUNCH_INDICES, k - j), st);
+            launch_res2d(G.shape, G.sims, G.nsims, c->h_launch + j, std::min(RES_LAUNCH_INDICES, k - j), st);
     }
     if (steps && no_graphs) {
         launch_steps(c, k, nra);

@@ -213,8 +213,7 @@ struct DevEntR {
     int sum;               // its partial sum, 0 .. 31
     double w;
 };
-struct DevRes2D {
-    DevSim2D s;
+struct DevRes {
     const DevResWarp *warps;   // [cluster rank][warp]
     const DevResCta *ctas;     // [cluster rank]
     const DevEntR *ents;
@@ -228,23 +227,34 @@ struct DevRes2D {
     int shift;                 // grid row of the cluster's first row (the grid is a torus)
     int np_max, ntile_max, ntile;   // pieces of a CTA at most, tiles (of any simulation, and of this one)
 };
+struct DevRes2D : DevRes {
+    DevSim2D s;
+};
+struct DevResCyl : DevRes {
+    DevSim6 s;
+};
 struct Res2dShape {
     int fp64, rb;          // rows of a thread's block
+    int cyl;               // 1: the cylindrical march (rescyl.cu)
     int cluster, threads, smem;
     int tcols, nb;
     int gen_words, stage_words, ne_max, shift;
     int np_max, npiece_max, ntile_max;
 };
-int res2d_words(int fp64, int rb, int *coef);   // 16-byte words of a thread's slots, and of its coefficients
+// 16-byte words of a thread's slots, and of its coefficients (returned in *coef)
+int res_words(int cyl, int fp64, int rb, int *coef);
+int rescyl_words(int fp64, int rb, int *coef);
+const void *rescyl_kernel(int fp64, int rb);   // rescyl.cu; null: no such variant
 constexpr int RES_CLUSTER_MAX = 16;
+constexpr int RES_MAXT = 512;                 // threads of a CTA: 128 registers a thread
 constexpr int RES_SMEM_MAX = 226 * 1024;      // dynamic shared memory of a CTA (the rest is static)
 constexpr int RES_LAUNCH_STEPS = 192;         // time steps of one launch at most (its weights sit in shared memory)
 constexpr int RES_LAUNCH_INDICES = RES_LAUNCH_STEPS / 3;
 cudaError_t res2d_prepare();
 int res2d_proj_bytes(const Res2dShape &q);      // shared memory of the projection's history and sums
-std::vector<Res2dShape> res2d_shapes(int fp64, int nx, int ny, int nsims);
+std::vector<Res2dShape> res2d_shapes(int cyl, int fp64, int nx, int ny, int nsims);
 // launch indices launch .. launch + count - 1
-void launch_res2d(const Res2dShape &q, const DevRes2D *sims, int nsims, int64_t launch, int count, cudaStream_t st);
+void launch_res2d(const Res2dShape &q, const void *sims, int nsims, int64_t launch, int count, cudaStream_t st);
 
 void launch_step2d(int fp64, const DevSim2D *sims, const DevTile *tiles, int ntiles,
                    const int64_t *launch_base, int64_t launch_add, cudaStream_t st);

@@ -26,93 +26,11 @@
 #include <cmath>
 #include <utility>
 
-#include "kernels.h"
+#include "resident.cuh"
 
 namespace cas {
 
 namespace {
-
-template <bool B>
-struct ResFlag {
-    static constexpr bool value = B;
-};
-
-template <typename R>
-struct Vec16 {
-    static constexpr int N = 16 / sizeof(R);
-    alignas(16) R c[N];
-};
-
-__device__ __forceinline__ unsigned cluster_rank()
-{
-    unsigned r;
-    asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ unsigned cluster_size()
-{
-    unsigned r;
-    asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-// full barrier of the cluster's threads (start and end of a launch; the steps use the mbarriers below)
-__device__ __forceinline__ void cluster_sync()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// shared::cluster address of this CTA's shared address `a` in the CTA of rank `r`
-__device__ __forceinline__ unsigned map_rank(unsigned a, unsigned r)
-{
-    unsigned o;
-    asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(o) : "r"(a), "r"(r));
-    return o;
-}
-// 16 bytes to another CTA of the cluster, counted on that CTA's mbarrier when they have landed
-__device__ __forceinline__ void st_async(unsigned a, unsigned mb, const Vec16<float> &v)
-{
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(a),
-                 "r"(__float_as_uint(v.c[0])), "r"(__float_as_uint(v.c[1])), "r"(__float_as_uint(v.c[2])), "r"(__float_as_uint(v.c[3])), "r"(mb)
-                 : "memory");
-}
-__device__ __forceinline__ void st_async(unsigned a, unsigned mb, const Vec16<double> &v)
-{
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];" ::"r"(a),
-                 "l"(__double_as_longlong(v.c[0])), "l"(__double_as_longlong(v.c[1])), "r"(mb)
-                 : "memory");
-}
-__device__ __forceinline__ void mb_init(unsigned mb, unsigned count) { asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mb), "r"(count) : "memory"); }
-__device__ __forceinline__ void mb_expect(unsigned mb, unsigned bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mb_try(unsigned mb, unsigned parity)
-{
-    unsigned ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2, 0x4000;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok)
-                 : "r"(mb), "r"(parity)
-                 : "memory");
-    return ok;
-}
-// Waits for the phase of the given parity; gives up after a second, which no correct run comes near, so
-// that the kernel always ends.
-__device__ __noinline__ bool mb_wait_long(unsigned mb, unsigned parity)
-{
-    unsigned long long t0, t1;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-    for (int i = 0; i < 1 << 26; ++i) {
-        if (mb_try(mb, parity)) return true;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
-        if (t1 - t0 > 1000000000ull) break;
-    }
-    return false;
-}
-__device__ __forceinline__ bool mb_wait(unsigned mb, unsigned parity)
-{
-    for (int i = 0; i < 64; ++i)
-        if (mb_try(mb, parity)) return true;
-    return mb_wait_long(mb, parity);
-}
 
 // A block's u depends on vx of the row above and vy of the column to the left.  RED (FP32): the thread
 // updates those itself as well, from the u around its block, so that one exchange of u per step is enough.
@@ -120,16 +38,6 @@ __device__ __forceinline__ bool mb_wait(unsigned mb, unsigned parity)
 // after V, and u after U.
 template <typename R>
 constexpr bool RES_RED = sizeof(R) == 4;
-
-// (double)v; a float's without the FP64 pipe, which takes 64 clocks for a warp's conversions
-__device__ __forceinline__ double widen(double v) { return v; }
-__device__ __forceinline__ double widen(float v)
-{
-    const unsigned b = __float_as_uint(v), m = b & 0x7fffffffu;
-    if (m - 0x00800000u < 0x7f000000u || m == 0u)   // normal, or zero
-        return __hiloint2double((int)((b & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)), (int)(b << 29));
-    return (double)v;
-}
 
 // 16-byte words of a thread's slots in shared memory, filled by its neighbours: a row from above (RED: u,
 // else vx), u of the row below, a column from the left (RED: u, else vy), u of the column to the right;
@@ -145,15 +53,6 @@ struct Slots {
     static constexpr int CVX = 0, CVY = RB + RED, CVYL = 2 * RB + RED, CU = 2 * RB + RED * (1 + KV);
     static constexpr int CWORDS = (3 * RB + RED * (1 + KV)) | 1;
 };
-
-// bits of the packed per-thread state
-constexpr unsigned F_ACTIVE = 1u, F_SHORT = 2u, F_FARU = 4u, F_FARD = 8u, F_NEEDU = 16u, F_NEEDD = 32u, F_LEADU = 64u, F_LEADD = 128u,
-                   F_LATE = 256u, F_STAGE = 512u, F_MINE = 1024u, F_DEAD = 2048u, F_FIRST = 4096u, F_STAGEW = 8192u;
-constexpr unsigned F_PLAIN = 1u << 23;
-constexpr int RES_WIN = 16;              // steps of a window of the projection
-constexpr int F_W = 14;                  // valid columns less one (2 bits)
-constexpr int F_ROWS = 16;               // staged rows of the block (7 bits)
-constexpr int F_CU = 24, F_CD = 28;      // CTAs of the bands above and below
 
 template <typename R, int RB, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1)
@@ -240,20 +139,16 @@ k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
     // in this order they round as before and do not depend on how the steps were cut into launches.
     const DevResWarp pw = D.warps[(int)rank * (nt >> 5) + warp];
     unsigned pk_stage;             // first staged word (16 bits), element of this thread's entry (16 bits)
-    const int stage_w = nt * SL::WORDS + D.gen_words, sbuf = D.stage_words, nem = D.ne_max;
-    const int np = D.ctas[rank].np, rounded = D.ctas[rank].rounded;
-    // behind the staged rows: this launch's weights, the entries' weights, partial sums, ..., the history
-    const int n_tail = S.tail_from + 1;                            // the first step of the tail's sums
-    const int gw_i = (stage_w + 2 * sbuf) * 2, we_i = gw_i + RES_LAUNCH_STEPS, ps_i = we_i + nem;
-    const int at_i = ps_i + D.np_max * 16 * RES_WIN;   // rank 0: the terms by tile and launch index
-    const int hist_i = (at_i + 2 * D.ntile_max * RES_LAUNCH_INDICES) * (int)(8 / sizeof(R));
-    double *const dd = reinterpret_cast<double *>(dyn);
+    const int stage_w = nt * SL::WORDS + D.gen_words, sbuf = D.stage_words;
+    ResSums<R> sums{reinterpret_cast<double *>(dyn), reinterpret_cast<double *>(S.fields) + D.term_off, slot, piece, n_lo, S.tail_from + 1,
+                    D.ctas[rank].np, D.ctas[rank].rounded};
+    sums.layout(stage_w + 2 * sbuf, D);
     {
         flags |= ((pw.lanes >> lane) & 1) ? F_STAGE : 0u;
         flags |= pw.lanes ? F_STAGEW : 0u;
         flags |= pw.rows << F_ROWS;
         const int st = stage_w + pw.stage0 + __popc(pw.lanes & ((1u << lane) - 1u)) * pw.stride;
-        for (int i = t; i < cnt; i += nt) dd[gw_i + i] = S.gw[n_lo - 1 + i];
+        for (int i = t; i < cnt; i += nt) sums.dd[sums.gw_i + i] = S.gw[n_lo - 1 + i];
         const DevResCta &pc = D.ctas[rank];
         int off = 0;
         for (int q = t; q < RES_PIECES * 32 + 1; q += nt) slot[q] = pc.slot[q];
@@ -261,7 +156,7 @@ k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
         if (t < pc.ne) {
             flags |= F_MINE;
             off = D.ents[pc.e0 + t].off;
-            dd[we_i + t] = D.ents[pc.e0 + t].w;
+            sums.dd[sums.we_i + t] = D.ents[pc.e0 + t].w;
         }
         pk_stage = (unsigned)st | (unsigned)off << 16;
     }
@@ -360,58 +255,8 @@ k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
             if ((flags & lead) && i + 2 < cnt) mb_expect(m, D.tcols * 16);
         }
     };
-    // Sums of the steps of window k that lie in [n_lo, last]: 32 partial sums a piece, added as a warp's shuffles
-    // add its lanes (on horizontal faces an entry's partial sum is its place in its row and the products are
-    // rounded, as in the other 2D kernels).  A half warp takes one partial sum, a lane of it one step; with
-    // entries in the first 16 alone, the halves take neighbouring ones.
-    auto part_sums = [&](int k, int last) {
-        const int ln = (int)threadIdx.x & 31, half = ln / RES_WIN, st = ln & (RES_WIN - 1), n = k * RES_WIN + st;
-        const R *const hs = reinterpret_cast<const R *>(dyn) + hist_i + (n & (2 * RES_WIN - 1)) * nem;
-        for (int pc = 0; pc < np; ++pc) {
-            const short *const sl = slot + 32 * pc;
-            const bool low = sl[16] == sl[32];
-            for (int q = (int)threadIdx.x >> 5; q < (low ? 8 : 16); q += (int)blockDim.x >> 5) {
-                double p = 0.0;
-                const int g = low ? 2 * q + half : q + 16 * half;
-                int e = sl[g];
-                const int e1 = sl[g + 1];
-                if (e < e1 && n >= n_lo && n <= last) {
-                    p = dd[we_i + e] * widen(hs[e]);
-                    if (rounded)
-                        for (++e; e < e1; ++e) p = __dadd_rn(p, __dmul_rn(dd[we_i + e], widen(hs[e])));
-                    else
-                        for (++e; e < e1; ++e) p = fma(dd[we_i + e], widen(hs[e]), p);
-                }
-                if (!low) p += __shfl_down_sync(0xffffffffu, p, RES_WIN);
-                if (low || half == 0) dd[ps_i + (pc * 16 + (g & 15)) * RES_WIN + st] = p;
-            }
-        }
-    };
-    auto add_window = [&](int k, int last) {   // by the last warps, after the barrier that follows part_sums
-        const int nw = (int)blockDim.x >> 5;
-        for (int pc = nw - 1 - ((int)threadIdx.x >> 5); pc < np; pc += nw) {
-            const int ln = (int)threadIdx.x & 31, half = ln / RES_WIN, st = ln & (RES_WIN - 1), n = k * RES_WIN + st;
-            const double *const ps = dd + ps_i + (pc * 16 + half) * RES_WIN + st;   // groups half, half + 2, ...
-            const double a0 = ps[0] + ps[8 * RES_WIN], a2 = ps[2 * RES_WIN] + ps[10 * RES_WIN];
-            const double a4 = ps[4 * RES_WIN] + ps[12 * RES_WIN], a6 = ps[6 * RES_WIN] + ps[14 * RES_WIN];
-            double s = (a0 + a4) + (a2 + a6);
-            s += __shfl_down_sync(0xffffffffu, s, RES_WIN);
-            if (half == 0 && n >= n_lo && n <= last)
-                reinterpret_cast<double *>(S.fields)[D.term_off + piece[pc] * RES_LAUNCH_STEPS + (n - n_lo)] = dd[gw_i + n - n_lo] * s;
-        }
-    };
-    // the entries' values of the launch's step i, staged before the last barrier, join the history; a window
-    // whose last step joined it before that barrier is summed, and added a step later (the same for every
-    // warp of the CTA)
     auto consume = [&](int i) {
-        const int n = n_lo + i;
-        if (flags & F_MINE)
-            reinterpret_cast<R *>(dyn)[hist_i + (n & (2 * RES_WIN - 1)) * nem + (int)threadIdx.x] =
-                reinterpret_cast<const R *>(blocks + stage_w + (i & 1) * sbuf)[pk_stage >> 16];
-        if (nem > 0 && (n & (RES_WIN - 2)) == 0) {
-            if ((n & 1) == 0 && i > 0) part_sums((n - 1) / RES_WIN, n - 1);
-            if ((n & 1) == 1 && i > 1) add_window((n - 2) / RES_WIN, n - 2);
-        }
+        sums.consume(i, flags & F_MINE, reinterpret_cast<const R *>(blocks + stage_w + (i & 1) * sbuf), (int)(pk_stage >> 16));
     };
     auto put_row = [&](unsigned far, int at, unsigned cta, unsigned mb, const V4 &v) {
         if (flags & far) st_async(map_rank((unsigned)__cvta_generic_to_shared(blocks + at), cta), map_rank(mb, cta), v);
@@ -751,68 +596,25 @@ k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
                     }
         }
     }
-    // the last window, and the one before it when its partial sums are the last thing consume() did
-    __syncthreads();
-    if (cnt > 1 && (n_hi & (RES_WIN - 1)) == 0) add_window((n_hi - 1) / RES_WIN, n_hi - 1);
-    __syncthreads();
-    part_sums(n_hi / RES_WIN, n_hi);
-    __syncthreads();
-    add_window(n_hi / RES_WIN, n_hi);
     if (dead) *D.status = 1;
-    // rank 0 adds the terms to the simulation's sums
-    const unsigned rk = cluster_rank();
-    if (cluster_size() > 1) {
-        __syncwarp();
-        cluster_sync();
-    } else {
-        __syncthreads();
-    }
-    if (rk != 0) return;
-    const int K = D.k, nt_ = D.ntile, total = (cnt + K - 1) / K * nt_;
-    const short *const tp = D.tile_pieces;
-    for (int x = t2; x < total; x += (int)blockDim.x) {
-        const int l = x / nt_, tl = x - l * nt_;
-        double c = 0.0, ct = 0.0;
-        for (int i = l * K; i < min(cnt, l * K + K); ++i) {
-            double cq = 0.0;
-            for (int p = tp[tl]; p < tp[tl + 1]; ++p) cq += reinterpret_cast<volatile const double *>(S.fields)[D.term_off + p * RES_LAUNCH_STEPS + i];
-            c += cq;
-            if (n_lo + i >= n_tail) ct += cq;
-        }
-        dd[at_i + x] = c;
-        dd[at_i + D.ntile_max * RES_LAUNCH_INDICES + x] = ct;
-    }
-    __syncthreads();
-    if (t2 == 0) {
-        double acc = *S.acc;
-#pragma unroll 8
-        for (int x = 0; x < total; ++x) acc += dd[at_i + x];
-        *S.acc = acc;
-    }
-    if (t2 == (int)blockDim.x - 1 && n_hi >= n_tail) {
-        double tail = *S.tail;
-#pragma unroll 8
-        for (int x = 0; x < total; ++x) tail += dd[at_i + D.ntile_max * RES_LAUNCH_INDICES + x];
-        *S.tail = tail;
-    }
+    sums.finish(D, cnt, S.acc, S.tail);
 }
 
 }  // namespace
 
-// threads per CTA at most: 128 registers a thread, of which RB * CX * 3 hold fields
-constexpr int RES_MAXT = 512;
-
 template <typename R, int RB>
 static const void *res2d_fn() { return (const void *)k_res2d<R, RB, RES_MAXT>; }
 
-static const void *res2d_kernel(int fp64, int rb)
+static const void *res_kernel(int cyl, int fp64, int rb)
 {
+    if (cyl) return rescyl_kernel(fp64, rb);
     if (fp64) return rb == 1 ? res2d_fn<double, 1>() : rb == 2 ? res2d_fn<double, 2>() : rb == 4 ? res2d_fn<double, 4>() : nullptr;
     return rb == 2 ? res2d_fn<float, 2>() : rb == 4 ? res2d_fn<float, 4>() : nullptr;
 }
 
-int res2d_words(int fp64, int rb, int *coef)   // Slots<R, rb>::WORDS, CWORDS
+int res_words(int cyl, int fp64, int rb, int *coef)   // Slots<R, rb>::WORDS, CWORDS
 {
+    if (cyl) return rescyl_words(fp64, rb, coef);
     const int cx = fp64 ? 2 : 4, kv = (rb + cx - 1) / cx, red = fp64 ? 0 : 1;
     *coef = (3 * rb + red * (1 + kv)) | 1;
     return ((1 + red) * (2 + 2 * kv)) | 1;
@@ -827,9 +629,9 @@ int res2d_proj_bytes(const Res2dShape &q)
 
 cudaError_t res2d_prepare()
 {
-    for (int f = 0; f < 2; ++f)
-        for (int rb : {1, 2, 4}) {
-            const void *k = res2d_kernel(f, rb);
+    for (int f = 0; f < 4; ++f)
+        for (int rb : {1, 2, 3, 4}) {
+            const void *k = res_kernel(f >> 1, f & 1, rb);
             if (!k) continue;
             cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RES_SMEM_MAX);
             if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -855,12 +657,12 @@ static cudaError_t launch_cfg(const void *k, int grid, int cluster, int threads,
     return k ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-void launch_res2d(const Res2dShape &q, const DevRes2D *sims, int nsims, int64_t launch, int count, cudaStream_t st)
+void launch_res2d(const Res2dShape &q, const void *sims, int nsims, int64_t launch, int count, cudaStream_t st)
 {
     if (nsims <= 0) return;
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at;
-    const void *k = res2d_kernel(q.fp64, q.rb);
+    const void *k = res_kernel(q.cyl, q.fp64, q.rb);
     if (launch_cfg(k, nsims * q.cluster, q.cluster, q.threads, q.smem, st, &cfg, &at) != cudaSuccess) return;
     void *args[] = {(void *)&sims, (void *)&launch, (void *)&count};
     cudaLaunchKernelExC(&cfg, k, args);
@@ -887,13 +689,13 @@ static int clusters_resident(const void *k, const Res2dShape &q, bool alone)
 // at once run one after the other.  Measured in FP32 (Gcell-updates/s, 400 x 166 cells, 640 simulations):
 // 4 rows in clusters of 9: 870, of 10: 749; 6 and 7 rows: 700 at most (fewer threads fit the shared
 // memory); the three-step kernel 465.  Larger grids than a cluster of 16 holds stay with that kernel.
-std::vector<Res2dShape> res2d_shapes(int fp64, int nx, int ny, int nsims)
+std::vector<Res2dShape> res2d_shapes(int cyl, int fp64, int nx, int ny, int nsims)
 {
     std::vector<std::pair<double, Res2dShape>> found;
     const int cx = fp64 ? 2 : 4;
     const int tcols = (nx + cx - 1) / cx;
-    for (int rb : {1, 2, 4}) {
-        const void *k = res2d_kernel(fp64, rb);
+    for (int rb : {1, 2, 3, 4}) {
+        const void *k = res_kernel(cyl, fp64, rb);
         if (!k) continue;
         const int nb = (ny + rb - 1) / rb;                       // bands of rb or rb - 1 rows
         if (rb > 1 && ny / nb < rb - 1) continue;
@@ -902,13 +704,14 @@ std::vector<Res2dShape> res2d_shapes(int fp64, int nx, int ny, int nsims)
             if (threads > RES_MAXT) continue;
             Res2dShape q{};
             q.fp64 = fp64;
+            q.cyl = cyl;
             q.rb = rb;
             q.cluster = c;
             q.threads = threads;
             q.tcols = tcols;
             q.nb = nb;
             int cw = 0;
-            q.smem = threads * res2d_words(fp64, rb, &cw) * 16 + RES_LAUNCH_STEPS * 8;
+            q.smem = (threads * res_words(cyl, fp64, rb, &cw) + (cyl ? 8 * tcols : 0)) * 16 + RES_LAUNCH_STEPS * 8;   // (cyl: radial factors)
             if (q.smem > RES_SMEM_MAX) continue;
             const int fit1 = clusters_resident(k, q, true), fit = std::max(fit1, clusters_resident(k, q, false));
             if (fit1 < 1) continue;
@@ -916,7 +719,9 @@ std::vector<Res2dShape> res2d_shapes(int fp64, int nx, int ny, int nsims)
             const int waves = (nsims + fit1 * share - 1) / (fit1 * share);
             const double warps = share * (threads / 32);
             double t;
-            if (fp64) {
+            if (cyl) {   // about 60 operations a cell
+                t = fp64 ? 1.22 * warps * 16.0 * rb * cx * 40.0 + 1000.0 : std::max(c > 1 ? 2500.0 : 2000.0, warps / 4.0 * (rb * cx * 60.0 + 200.0) * 1.6);
+            } else if (fp64) {
                 t = 1.22 * warps * 16.0 * rb * cx * 9.0 + 700.0;
             } else {
                 const double chain = c > 1 ? 1750.0 : 1200.0, issue = (rb == 4 ? 137.0 : 120.0) * warps;

@@ -97,6 +97,31 @@ def test_resident_pmc_and_many_materials(ctx):
     _compare(ctx, _box(90, 47, "fp64", 250, objects=objs))
 
 
+def _cylinder(resolution, h, m_list, prec, steps):
+    p = W.cylinder_blocks(h, resolution=resolution, m_list=m_list, n_harm=2, precision=prec)
+    p["n_steps"] = steps
+    return p
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("resolution,h,m_list,steps", [(10, 0.5, (0, 1), 150), (14, 0.5, (1, 2), 129), (18, 1.0, (0, 2), 256),
+                                                        (24, 2.0, (0, 1, 2), 130), (40, 1.0, (1,), 65)])
+def test_resident_cylinder_equals_two_step_march(ctx, prec, resolution, h, m_list, steps):
+    p = _cylinder(resolution, h, m_list, prec, steps)
+    _, per, st = ctx.plan(p).run(per_sim=True)
+    _, per2, _ = ctx.plan(p, options={"steps_per_launch": 2}).run(per_sim=True)
+    lim = 16 * 2.0 ** -53 * np.sqrt(steps) * np.max(np.abs(per2))
+    assert np.max(np.abs(per - per2)) <= lim, np.max(np.abs(per - per2)) / lim
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_resident_cylinder_against_oracle(ctx, prec):
+    p = _cylinder(10, 0.5, (0, 1, 2), prec, 120)
+    F, per, _ = ctx.plan(p).run(per_sim=True)
+    Fo, parts, _ = oracle.force(p, return_parts=True)
+    assert_parity(per, F[p["force_axis"]], np.array(parts), Fo, p["n_steps"], prec == "fp64", "cylinder")
+
+
 def test_resident_results_do_not_depend_on_the_batch(ctx):
     probs = [_box(66, 50, "fp32", 301), _box(83, 45, "fp64", 250), _box(66, 50, "fp32", 500), _box(130, 40, "fp32", 333)]
     alone = [ctx.plan(p).run()[0] for p in probs]
