@@ -157,7 +157,17 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
         return gen.emplace(geo, std::move(g)).first->second;
     };
     std::vector<DevResWarp> rec((size_t)q->cluster * nwarp);
-    for (const Sim &sm : D.sims) {
+    // The harmonics of a face share their sites: a simulation measured at the sites of an earlier one of its
+    // lattice, face and source component takes that one's tables with its own weights.
+    struct Like {
+        size_t sim;                   // the earlier simulation
+        int64_t e0;                   // its first entry
+        std::vector<Entry> meas;
+        std::vector<int> from;        // entry -> place in meas
+    };
+    std::map<std::array<int, 4>, Like> like;
+    for (size_t si = 0; si < D.sims.size(); ++si) {
+        const Sim &sm = D.sims[si];
         std::fill(rec.begin(), rec.end(), DevResWarp{});
         const int arrays = q->cyl ? 3 : (sm.second_u ? 1 : 2);
         // the sigma group's first array; cylindrical: the entries of the source's real set alone (prepare_plan)
@@ -166,6 +176,24 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
         std::vector<Entry> meas;
         for (const Entry &e : sm.meas)
             if (!q->cyl || sm.src.empty() || in_a(e.arr) == in_a(sm.src[0].arr)) meas.push_back(e);
+        const std::array<int, 4> key{sm.geo, sm.face, sm.kind, sm.comp};
+        auto lk = like.find(key);
+        if (lk != like.end() && D.sims[lk->second.sim].second_u == sm.second_u && lk->second.meas.size() == meas.size() &&
+            std::equal(meas.begin(), meas.end(), lk->second.meas.begin(), [](const Entry &x, const Entry &y) { return x.arr == y.arr && x.idx == y.idx; })) {
+            const Like &l = lk->second;
+            const size_t nw = rec.size(), nc = (size_t)q->cluster;
+            for (size_t v = 0; v < nw; ++v) P->resW.push_back(P->resW[l.sim * nw + v]);
+            for (size_t v = 0; v < nc; ++v) P->resC.push_back(P->resC[l.sim * nc + v]);
+            for (size_t v = 0; v <= RES_TILES; ++v) P->resT.push_back(P->resT[l.sim * (RES_TILES + 1) + v]);
+            P->resNT.push_back(P->resNT[l.sim]);
+            for (size_t v = 0; v < l.from.size(); ++v) {
+                DevEntR en = P->resE[(size_t)l.e0 + v];
+                en.w = meas[l.from[v]].re;
+                P->resE.push_back(en);
+            }
+            continue;
+        }
+        Like made{si, (int64_t)P->resE.size(), meas, {}};
         // the place of an entry: CTA, warp record, lane, row and element of the block
         auto place = [&](const Entry &e, int *cta, int *lane, int *row, int *el) -> DevResWarp & {
             const int i = (int)(e.idx % nx), j = (int)((e.idx / nx - q->shift + ny) % ny);   // the cluster's row
@@ -217,7 +245,7 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
             const DevResWarp &w = place(e, &cta, &lane, &row, &el);
             const int word = w.stage0 + __builtin_popcount(w.lanes & ((1u << lane) - 1u)) * w.stride +
                              __builtin_popcount(w.rows & ((1u << row) - 1u)) * arrays + e.arr - arr0;
-            byp[cta].push_back({tile, DevEntR{word * cx + el, sum, e.re}});
+            byp[cta].push_back({tile, DevEntR{word * cx + el, sum, (double)(&e - meas.data())}});   // its place, until the order is known
             pieces[{tile, cta}] = 0;
         }
         short tp[RES_TILES + 1] = {};
@@ -261,9 +289,13 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
             }
             q->np_max = std::max(q->np_max, (int)rc.np);
             P->resC.push_back(rc);
-            for (const auto &be : b) P->resE.push_back(be.second);
+            for (const auto &be : b) {
+                made.from.push_back((int)be.second.w);
+                P->resE.push_back(DevEntR{be.second.off, be.second.sum, meas[(size_t)made.from.back()].re});
+            }
         }
         P->resW.insert(P->resW.end(), rec.begin(), rec.end());
+        like[key] = std::move(made);
     }
     if ((int64_t)q->npiece_max * RES_LAUNCH_STEPS * 8 + 8 > (q->cyl ? 6 : 3) * (int64_t)nx * ny * (int64_t)P->rsize) return false;   // their terms wait in the second field buffer
     q->gen_words = gen_max * 32 * cwords;

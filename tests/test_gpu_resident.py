@@ -58,7 +58,7 @@ def _compare(ctx, p):
     return F, per
 
 
-SIZES = [(2, 7), (3, 12), (5, 1), (9, 2), (33, 13), (64, 64), (61, 29), (83, 45), (130, 7), (400, 83), (251, 93), (127, 201), (512, 130)]
+SIZES = [(2, 7), (3, 12), (5, 1), (9, 2), (33, 13), (64, 64), (61, 29), (83, 45), (130, 7), (400, 83), (251, 93), (127, 201), (512, 130), (500, 201)]
 
 
 @pytest.mark.parametrize("prec", ["fp32", "fp64"])
