@@ -8,8 +8,9 @@
 // Layout: a thread owns a block of CX columns (16 bytes) by RB rows of u, vx, vy in registers;
 // `tcols` threads cover a row band of the grid, bands are RB or RB - 1 rows high, and the bands
 // are dealt to the cluster's CTAs in order, from grid row `shift` on (so that no CTA boundary parts the
-// rows of a horizontal face, whose functional may cancel along it and is summed step by step in one CTA).  The grid is a torus (closed walls are masked sites),
-// so the first band's upper neighbour is the last band.  Per step
+// rows of a horizontal face, whose functional may cancel along it and is summed step by step in one CTA).
+// The grid is a torus (closed walls are masked sites), so the first band's upper neighbour is the last
+// band.  Per step
 //   V: vx(r) from u(r + 1) - u(r), vy(c) from u(c + 1) - u(c)
 //   U: u from vy(c) - vy(c - 1) and vx(r) - vx(r - 1)
 // (sigma on u: V then U; sigma on v: U then V, run as U, (V, U), ..., V).  A thread updates vx of the row
@@ -20,6 +21,13 @@
 // previous CTA goes by st.async, which counts its bytes on that CTA's mbarrier; only the warps of the
 // band that needs it wait there.  Two buffers of slots by step parity: a neighbour writes the slots of
 // step n + 2 only after the barrier that follows this thread's reads of step n.
+//
+// Bound by the chain of one step (slots, barrier, far rows) on small grids and by that and issue on large
+// ones (16 warps of 128 registers on an SM, 52% of the issue slots); memory holds the fields only between
+// launches of up to 192 steps.  Measured against the multi-step kernels, whose fields pass through memory
+// every two or three steps (Gcell-updates/s): FP32 400 x 166, 640 simulations 465 -> 779; 128 x 128, 80
+// simulations 734, 64 x 64, 40 simulations 514, 32 x 16 155; whole FP64 plate forces 88.5 -> 8.3 ms, FP64
+// 251 x 93 44.5 -> 24.6 ms.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -133,10 +141,11 @@ k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
     // of RES_WIN steps, and every RES_WIN steps the CTA forms s(n) = sum_e w_e F_e(n) of the window's steps,
     // one lane per step and group of entries (in FP64; GB300's FP64 pipe takes 64 clocks per warp
     // instruction, which a reduction per step put on the critical path of every step).
-    // The terms w_n s(n) go to the second field buffer (unused otherwise), and rank 0 adds them at the end of the launch as the multi-step kernels do: by
-    // tile and launch index (a CTA's entries of one tile are a piece).  The sum over a run's steps is rounded
-    // to the last bit of its early terms thousands of times, the force is a small difference of such sums, and
-    // in this order they round as before and do not depend on how the steps were cut into launches.
+    // The terms w_n s(n) go to the second field buffer (unused otherwise), and rank 0 adds them at the end of
+    // the launch as the multi-step kernels do: by tile and launch index (a CTA's entries of one tile are a
+    // piece).  The sum over a run's steps is rounded to the last bit of its early terms thousands of times, the
+    // force is a small difference of such sums, and in this order they round as before and do not depend on
+    // how the steps were cut into launches.
     const DevResWarp pw = D.warps[(int)rank * (nt >> 5) + warp];
     unsigned pk_stage;             // first staged word (16 bits), element of this thread's entry (16 bits)
     const int stage_w = nt * SL::WORDS + D.gen_words, sbuf = D.stage_words;
@@ -167,7 +176,7 @@ k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
     // step2d_tk.cu); the half step at n = 1 halves the first group
     R u[RB][CX], vx[RB][CX], vy[RB][CX], vxm[RED ? CX : 1], vym[RED ? RB : 1];   // vxm, vym with RED only
     const bool su = S.second_u != 0;
-    R cxu, cyu, cuu;   // the coefficients of a warp whose cells are all of one material
+    R cxu, cyu, cuu;   // the coefficients of a warp whose cells are all of one material (those of vx negated, here and in the tables)
     const bool uni = pw.gen < 0;
     const V4 *const ow = blocks + nt * SL::WORDS + ((uni ? 0 : pw.gen) * 32 + lane) * SL::CWORDS;
     {
@@ -196,7 +205,7 @@ k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
                     const unsigned g = (unsigned)(grid_row(y0 + r) * nx + x0 + c);
                     vvx = fvx[g];
                     const int m = mat[g];
-                    kx.c[c] = fV * coef[3 * m + 1];
+                    kx.c[c] = -fV * coef[3 * m + 1];
                     if (r >= 0) {
                         vu = fu[g];
                         vvy = fvy[g];
@@ -241,7 +250,7 @@ k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
         int m0 = active ? mat[(unsigned)(grid_row(y0) * nx + x0)] : 0;
         m0 = __shfl_sync(0xffffffffu, m0, act ? __ffs(act) - 1 : 0);
         cuu = fU * coef[3 * m0];
-        cxu = fV * coef[3 * m0 + 1];
+        cxu = -fV * coef[3 * m0 + 1];
         cyu = fV * coef[3 * m0 + 2];
     }
     const R a = (R)S.a;
@@ -343,9 +352,28 @@ k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
             if constexpr (UNI) return arr == 1 ? cyu : cuu;
             else return reinterpret_cast<const R *>(ow + (arr == 1 ? SL::CVY : SL::CU) + r)[c];
         };
-        auto upx = [&](R v, R k, R d) -> R { return SU ? v - k * d : a * v - k * d; };
+        auto upx = [&](R v, R k, R d) -> R { return SU ? v + k * d : a * v + k * d; };   // k is negated
         auto upy = [&](R v, R k, R d) -> R { return SU ? v + k * d : a * v + k * d; };
         auto upu = [&](R v, R k, R d) -> R { return SU ? a * v + k * d : v + k * d; };
+        // vx of a row from u of the row below it (`hi`) and its own (`lo`).  FP32 takes two cells per instruction,
+        // with the operations and roundings of one at a time (x - y as y * -1 + x): 7.39 -> 7.15 us a step at
+        // 128 x 128 (40 simulations), 757.8 -> 779.3 Gcell-updates/s on the 400 x 166 sweep.  u in pairs as well: 777.1,
+        // and 0.747 -> 0.790 us a step on grids of a few warps (its differences along x are no aligned pairs).
+        auto row_vx = [&](R (&f)[CX], const V4 &k, const R *hi, const R *lo) {
+            if constexpr (sizeof(R) == 4) {
+#pragma unroll
+                for (int c = 0; c < CX; c += 2) {
+                    const float2 v = make_float2(f[c], f[c + 1]), kk = make_float2(k.c[c], k.c[c + 1]);
+                    const float2 d = __ffma2_rn(make_float2(lo[c], lo[c + 1]), make_float2(-1.0f, -1.0f), make_float2(hi[c], hi[c + 1]));
+                    const float2 o = SU ? __ffma2_rn(kk, d, v) : __ffma2_rn(make_float2(a, a), v, __fmul2_rn(kk, d));
+                    f[c] = o.x;
+                    f[c + 1] = o.y;
+                }
+            } else {
+#pragma unroll
+                for (int c = 0; c < CX; ++c) f[c] = upx(f[c], k.c[c], hi[c] - lo[c]);
+            }
+        };
         auto stage = [&](int i) {
             if (flags & F_STAGE) {
                 V4 *q = blocks + (pk_stage & 0xffffu) + (i & 1) * sbuf;
@@ -383,8 +411,7 @@ k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
         auto v_up = [&](const V4 *own) {
             if constexpr (RED) {
                 const V4 hu = own[SL::UP], k = row(0, -1);
-#pragma unroll
-                for (int c = 0; c < CX; ++c) vxm[RED ? c : 0] = upx(vxm[RED ? c : 0], k.c[c], u[0][c] - hu.c[c]);
+                row_vx(vxm, k, u[0], hu.c);
             }
         };
         // vx of the last rows from u of the row below
@@ -396,13 +423,10 @@ k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
 #pragma unroll
                 for (int c = 0; c < CX; ++c) u[RB - 1][c] = cut ? hd.c[c] : u[RB - 1][c];
                 const V4 k = row(0, RB > 1 ? RB - 2 : 0);
-#pragma unroll
-                for (int c = 0; c < CX; ++c)
-                    vx[RB > 1 ? RB - 2 : 0][c] = upx(vx[RB > 1 ? RB - 2 : 0][c], k.c[c], u[RB - 1][c] - u[RB > 1 ? RB - 2 : 0][c]);
+                row_vx(vx[RB > 1 ? RB - 2 : 0], k, u[RB - 1], u[RB > 1 ? RB - 2 : 0]);
             }
             const V4 k = row(0, RB - 1);
-#pragma unroll
-            for (int c = 0; c < CX; ++c) vx[RB - 1][c] = upx(vx[RB - 1][c], k.c[c], hd.c[c] - u[RB - 1][c]);
+            row_vx(vx[RB - 1], k, hd.c, u[RB - 1]);
         };
         // V phase: the part no neighbour's u enters, the step's barrier, the columns at the sides (RED), the rest
         auto phase_v = [&](int i) {
@@ -426,8 +450,7 @@ k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
                 }
                 if (r + 2 < RB) {
                     const V4 k = row(0, r);
-#pragma unroll
-                    for (int c = 0; c < CX; ++c) vx[r][c] = upx(vx[r][c], k.c[c], u[r + 1][c] - u[r][c]);
+                    row_vx(vx[r], k, u[r + 1], u[r]);
                 }
             }
             if (!(flags & F_LATE)) __syncthreads();
@@ -686,9 +709,10 @@ static int clusters_resident(const void *k, const Res2dShape &q, bool alone)
 // for the warps that share an SM: FP32 the larger of 137 a warp (measured with 16 warps; 307 instructions
 // a warp, 52% of the issue slots) and of one warp's own chain (1200; 1750 when rows come from other CTAs);
 // FP64 its arithmetic at two lanes a clock and SM times 1.22, plus 700.  Simulations beyond those resident
-// at once run one after the other.  Measured in FP32 (Gcell-updates/s, 400 x 166 cells, 640 simulations):
-// 4 rows in clusters of 9: 870, of 10: 749; 6 and 7 rows: 700 at most (fewer threads fit the shared
-// memory); the three-step kernel 465.  Larger grids than a cluster of 16 holds stay with that kernel.
+// at once run one after the other.  Measured in FP32 (Gcell-updates/s, 400 x 166 cells, 640 simulations,
+// without the projection, which costs 13%): 4 rows in clusters of 9: 870, of 10: 749; 6 and 7 rows: 700 at
+// most (fewer threads fit the shared memory); the three-step kernel 465 with its projection.  Grids larger
+// than a cluster of 16 holds stay with that kernel, at 539 on 512 x 512.
 std::vector<Res2dShape> res2d_shapes(int cyl, int fp64, int nx, int ny, int nsims)
 {
     std::vector<std::pair<double, Res2dShape>> found;
