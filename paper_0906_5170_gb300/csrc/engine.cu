@@ -300,7 +300,7 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
     if ((int64_t)q->npiece_max * RES_LAUNCH_STEPS * 8 + 8 > (q->cyl ? 6 : 3) * (int64_t)nx * ny * (int64_t)P->rsize) return false;   // their terms wait in the second field buffer
     q->gen_words = gen_max * 32 * cwords;
     q->smem += 16 * (q->gen_words + 2 * q->stage_words) + res2d_proj_bytes(*q);   // (the radial factors are in smem already)
-    if (nwarp * 32 * res_words(q->cyl, q->fp64, q->rb, &cwords) + q->gen_words + 8 * q->tcols + 2 * q->stage_words >= 1 << 16) return false;   // packed into 16 bits
+    if (nwarp * 32 * res_words(q->cyl, q->fp64, q->rb, &cwords) + q->gen_words + RES_RAD * q->tcols + 2 * q->stage_words >= 1 << 16) return false;   // packed into 16 bits
     return q->smem <= RES_SMEM_MAX;
 }
 

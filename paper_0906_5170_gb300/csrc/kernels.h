@@ -247,6 +247,7 @@ int rescyl_words(int fp64, int rb, int *coef);
 const void *rescyl_kernel(int fp64, int rb);   // rescyl.cu; null: no such variant
 constexpr int RES_CLUSTER_MAX = 16;
 constexpr int RES_MAXT = 512;                 // threads of a CTA: 128 registers a thread
+constexpr int RES_RAD = 9;                    // 16-byte words between the radial factors of two thread columns (8 of them; odd: no bank conflicts)
 constexpr int RES_SMEM_MAX = 226 * 1024;      // dynamic shared memory of a CTA (the rest is static)
 constexpr int RES_LAUNCH_STEPS = 192;         // time steps of one launch at most (its weights sit in shared memory)
 constexpr int RES_LAUNCH_INDICES = RES_LAUNCH_STEPS / 3;

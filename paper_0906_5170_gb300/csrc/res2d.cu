@@ -712,7 +712,9 @@ static int clusters_resident(const void *k, const Res2dShape &q, bool alone)
 // at once run one after the other.  Measured in FP32 (Gcell-updates/s, 400 x 166 cells, 640 simulations,
 // without the projection, which costs 13%): 4 rows in clusters of 9: 870, of 10: 749; 6 and 7 rows: 700 at
 // most (fewer threads fit the shared memory); the three-step kernel 465 with its projection.  Grids larger
-// than a cluster of 16 holds stay with that kernel, at 539 on 512 x 512.
+// than a cluster of 16 holds stay with that kernel, at 539 on 512 x 512.  Cylindrical, FP32: 27.5 clocks a
+// warp and cell of a thread (29 with three rows, which spill a little) and 770, at least 2300; 126 simulations of
+// 60 x 400: two rows in clusters of 6 229 Gcell-updates/s, of 7 177, of 9 202, three rows in clusters of 5 220, of 6 224.
 std::vector<Res2dShape> res2d_shapes(int cyl, int fp64, int nx, int ny, int nsims)
 {
     std::vector<std::pair<double, Res2dShape>> found;
@@ -735,7 +737,7 @@ std::vector<Res2dShape> res2d_shapes(int cyl, int fp64, int nx, int ny, int nsim
             q.tcols = tcols;
             q.nb = nb;
             int cw = 0;
-            q.smem = (threads * res_words(cyl, fp64, rb, &cw) + (cyl ? 8 * tcols : 0)) * 16 + RES_LAUNCH_STEPS * 8;   // (cyl: radial factors)
+            q.smem = (threads * res_words(cyl, fp64, rb, &cw) + (cyl ? RES_RAD * tcols : 0)) * 16 + RES_LAUNCH_STEPS * 8;   // (cyl: radial factors)
             if (q.smem > RES_SMEM_MAX) continue;
             const int fit1 = clusters_resident(k, q, true), fit = std::max(fit1, clusters_resident(k, q, false));
             if (fit1 < 1) continue;
@@ -743,8 +745,8 @@ std::vector<Res2dShape> res2d_shapes(int cyl, int fp64, int nx, int ny, int nsim
             const int waves = (nsims + fit1 * share - 1) / (fit1 * share);
             const double warps = share * (threads / 32);
             double t;
-            if (cyl) {   // about 60 operations a cell
-                t = fp64 ? 1.22 * warps * 16.0 * rb * cx * 40.0 + 1000.0 : std::max(c > 1 ? 2500.0 : 2000.0, warps / 4.0 * (rb * cx * 60.0 + 200.0) * 1.6);
+            if (cyl) {
+                t = fp64 ? 1.22 * warps * 16.0 * rb * cx * 40.0 + 1000.0 : std::max(2300.0, warps * rb * cx * (rb == 3 ? 29.0 : 27.5) + 770.0);
             } else if (fp64) {
                 t = 1.22 * warps * 16.0 * rb * cx * 9.0 + 700.0;
             } else {

@@ -11,8 +11,8 @@
 // neighbours' slots; the cells that need no neighbour come before the phase's barrier, the others after it.
 //
 // Bound by the latency of one warp's chain and its two barriers a step rather than by memory: 126
-// simulations of 60 x 400 cells run at 115 Gcell-updates/s in FP32 (72 with two steps per launch through
-// memory), in FP64 at 13.4 (4.5).
+// simulations of 60 x 400 cells run at 229 Gcell-updates/s in FP32 (72 with two steps per launch through
+// memory; 115 while the radial factors' loads met in the same banks), in FP64 at 13.4 (4.5).
 #include "resident.cuh"
 
 namespace cas {
@@ -97,7 +97,7 @@ k_rescyl(const DevResCyl *__restrict__ sims, int64_t launch, int count)
     // projection of the sigma group, as in res2d.cu (three components a staged row)
     const DevResWarp pw = D.warps[(int)rank * (nt >> 5) + warp];
     unsigned pk_stage;
-    const int stage_w = nt * SL::WORDS + D.gen_words + 8 * tcols, sbuf = D.stage_words;
+    const int stage_w = nt * SL::WORDS + D.gen_words + RES_RAD * tcols, sbuf = D.stage_words;
     ResSums<R> sums{reinterpret_cast<double *>(dyn), reinterpret_cast<double *>(S.fields) + D.term_off, slot, piece, n_lo, S.tail_from + 1,
                     D.ctas[rank].np, D.ctas[rank].rounded};
     sums.layout(stage_w + 2 * sbuf, D);
@@ -118,7 +118,8 @@ k_rescyl(const DevResCyl *__restrict__ sims, int64_t launch, int count)
         pk_stage = (unsigned)st | (unsigned)off << 16;
     }
 
-    // radial factors of the CTA's columns (step6c2.cu's, with kA or kB where they enter): 8 rows of CX per thread column
+    // radial factors of the CTA's columns (step6c2.cu's, with kA or kB where they enter): 8 rows of CX per thread
+    // column, RES_RAD words apart (8 apart, all lanes of a load met in the same banks)
     const R bxr = (R)S.bre[0], idx = (R)S.inv_dx;
     V4 *const rad = blocks + nt * SL::WORDS + D.gen_words;
     for (int q = t; q < tcols; q += nt) {
@@ -139,9 +140,9 @@ k_rescyl(const DevResCyl *__restrict__ sims, int64_t launch, int count)
             f[7].c[c] = col > 0 ? (ci - (R)0.5) / ci : (R)0;             // fb
         }
 #pragma unroll
-        for (int k = 0; k < 8; ++k) rad[q * 8 + k] = f[k];
+        for (int k = 0; k < 8; ++k) rad[q * RES_RAD + k] = f[k];
     }
-    const V4 *const my_rad = rad + tc * 8;
+    const V4 *const my_rad = rad + tc * RES_RAD;
 
     R e[3][RB][CX], hh[3][RB][CX];
     const bool electric = S.magnetic == 0;
@@ -351,10 +352,18 @@ k_rescyl(const DevResCyl *__restrict__ sims, int64_t launch, int count)
                 }
             }
         };
+        auto read_cols = [](const V4 *from, R (&to)[2 * KV * CX]) {   // two columns, by 16-byte loads
+#pragma unroll
+            for (int k = 0; k < 2 * KV; ++k) {
+                const V4 v = from[k];
+#pragma unroll
+                for (int c = 0; c < CX; ++c) to[k * CX + c] = v.c[c];
+            }
+        };
         auto phase_h = [&](int i) {
-            const R *const er = reinterpret_cast<const R *>(own + SL::ER);
             if (flags & F_LATE) {   // the ragged right edge keeps the column across the wall in its first unused one
                 __syncthreads();
+                const R *const er = reinterpret_cast<const R *>(own + SL::ER);
                 const int w = (int)((flags >> F_W) & 3u) + 1;
 #pragma unroll
                 for (int r = 0; r < RB; ++r)
@@ -367,11 +376,13 @@ k_rescyl(const DevResCyl *__restrict__ sims, int64_t launch, int count)
             }
             V4 z{};
 #pragma unroll
-            for (int r = 0; r + 2 < RB; ++r) rows_h(r, true, false, z, z, er);
+            for (int r = 0; r + 2 < RB; ++r) rows_h(r, true, false, z, z, nullptr);
             if (!(flags & F_LATE)) __syncthreads();
             if (EL && i > 0) consume(i - 1);
             wait_far(F_NEEDD, F_LEADD, mb_d, i);
             const V4 ed0 = own[SL::ED], ed2 = own[SL::ED + 1];
+            R er[2 * KV * CX];
+            read_cols(own + SL::ER, er);
             if (RB > 1) {
                 const bool cut = flags & F_SHORT;
 #pragma unroll
@@ -397,14 +408,15 @@ k_rescyl(const DevResCyl *__restrict__ sims, int64_t launch, int count)
             }
         };
         auto phase_e = [&](int i) {
-            const R *const hl = reinterpret_cast<const R *>(own + SL::HL);
             V4 z{};
 #pragma unroll
-            for (int r = 1; r < RB; ++r) rows_e(r, true, false, z, z, hl);
+            for (int r = 1; r < RB; ++r) rows_e(r, true, false, z, z, nullptr);
             __syncthreads();
             if (!EL && i > 0) consume(i - 1);
             wait_far(F_NEEDU, F_LEADU, mb_u, i);
             const V4 hu0 = own[SL::HU], hu2 = own[SL::HU + 1];
+            R hl[2 * KV * CX];
+            read_cols(own + SL::HL, hl);
 #pragma unroll
             for (int r = 0; r < RB; ++r) rows_e(r, false, true, hu0, hu2, hl);
         };
