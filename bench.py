@@ -36,6 +36,9 @@ DRAM_BYTES_PER_CELL_LAUNCH = {
     "k_step2d_tk<float, 3>": {"bytes_per_cell": (211.063e6 + 162.221e6) / 16998400,
                               "source": "paper_0906_5170_gb300/csrc/step2d_tk.cu", "sha256_16": "78d8356d7697ee99",
                               "profile": "profiles/k_step2d_tk_piston_sweep.md"},
+    "k_res2d<float>": {"bytes_per_cell": (206.963e6 + 150.095e6) / 16998400,
+                       "source": "paper_0906_5170_gb300/csrc/res2d.cu", "sha256_16": "efcf87a30f636a43",
+                       "profile": "profiles/k_res2d_piston_sweep.md"},
 }
 
 

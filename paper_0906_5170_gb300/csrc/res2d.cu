@@ -23,10 +23,10 @@
 // step n + 2 only after the barrier that follows this thread's reads of step n.
 //
 // Bound by the chain of one step (slots, barrier, far rows) on small grids and by that and issue on large
-// ones (16 warps of 128 registers on an SM, 52% of the issue slots); memory holds the fields only between
+// ones (16 warps of 128 registers on an SM, 45% of the issue slots); memory holds the fields only between
 // launches of up to 192 steps.  Measured against the multi-step kernels, whose fields pass through memory
-// every two or three steps (Gcell-updates/s): FP32 400 x 166, 640 simulations 465 -> 779; 128 x 128, 80
-// simulations 734, 64 x 64, 40 simulations 514, 32 x 16 155; whole FP64 plate forces 88.5 -> 8.3 ms, FP64
+// every two or three steps (Gcell-updates/s): FP32 400 x 166, 640 simulations 465 -> 779; 128 x 128, 320
+// simulations 734, 64 x 64, 160 simulations 514, 60 x 20, 96 simulations 155; whole FP64 plate forces 88.5 -> 8.3 ms, FP64
 // 251 x 93 44.5 -> 24.6 ms.
 #include <cuda_runtime.h>
 
@@ -357,7 +357,7 @@ k_res2d(const DevRes2D *__restrict__ sims, int64_t launch, int count)
         auto upu = [&](R v, R k, R d) -> R { return SU ? a * v + k * d : v + k * d; };
         // vx of a row from u of the row below it (`hi`) and its own (`lo`).  FP32 takes two cells per instruction,
         // with the operations and roundings of one at a time (x - y as y * -1 + x): 7.39 -> 7.15 us a step at
-        // 128 x 128 (40 simulations), 757.8 -> 779.3 Gcell-updates/s on the 400 x 166 sweep.  u in pairs as well: 777.1,
+        // 128 x 128 (320 simulations), 757.8 -> 779.3 Gcell-updates/s on the 400 x 166 sweep.  u in pairs as well: 777.1,
         // and 0.747 -> 0.790 us a step on grids of a few warps (its differences along x are no aligned pairs).
         auto row_vx = [&](R (&f)[CX], const V4 &k, const R *hi, const R *lo) {
             if constexpr (sizeof(R) == 4) {
@@ -706,13 +706,15 @@ static int clusters_resident(const void *k, const Res2dShape &q, bool alone)
 }
 
 // Shapes that hold an nx x ny simulation, the fastest by the model first.  The model's clocks of a step
-// for the warps that share an SM: FP32 the larger of 137 a warp (measured with 16 warps; 307 instructions
-// a warp, 52% of the issue slots) and of one warp's own chain (1200; 1750 when rows come from other CTAs);
+// for the warps that share an SM: FP32 the larger of 137 a warp (measured with 16 warps; about 300
+// instructions a warp, 45% of the issue slots) and of one warp's own chain (1200; 1750 when rows come from other CTAs);
 // FP64 its arithmetic at two lanes a clock and SM times 1.22, plus 700.  Simulations beyond those resident
 // at once run one after the other.  Measured in FP32 (Gcell-updates/s, 400 x 166 cells, 640 simulations,
 // without the projection, which costs 13%): 4 rows in clusters of 9: 870, of 10: 749; 6 and 7 rows: 700 at
 // most (fewer threads fit the shared memory); the three-step kernel 465 with its projection.  Grids larger
-// than a cluster of 16 holds stay with that kernel, at 539 on 512 x 512.  Cylindrical, FP32: 27.5 clocks a
+// than a cluster of 16 holds stay with that kernel, at 539 on 512 x 512 (256 simulations).  Every shape that
+// fits is taken: against the multi-step kernels the worst, clusters of 11 to 14 that leave a third of the SMs
+// idle, ran at 436 : 409 (FP32, 400 x 200, 320 simulations) and 30.1 : 28.5 (FP64, 256 x 200, 160).  Cylindrical, FP32: 27.5 clocks a
 // warp and cell of a thread (29 with three rows, which spill a little) and 770, at least 2300; 126 simulations of
 // 60 x 400: two rows in clusters of 6 229 Gcell-updates/s, of 7 177, of 9 202, three rows in clusters of 5 220, of 6 224.
 std::vector<Res2dShape> res2d_shapes(int cyl, int fp64, int nx, int ny, int nsims)
