@@ -2171,6 +2171,8 @@ int casimir_submit(casimir_plan_t *P, uint64_t tag, casimir_ticket *out)
     if (c->sync_busy.load()) return fail(CASIMIR_EBUSY, "a synchronous run is using the context");
     auto *r = new casimir_request();
     r->plan = P;
+    r->ctx = c;
+    r->cell_updates = P->cells * (int64_t)P->data.prob.n_steps;
     r->tag = tag;
     r->t_submit = now_ms();
     {
@@ -2190,7 +2192,7 @@ int casimir_submit(casimir_plan_t *P, uint64_t tag, casimir_ticket *out)
 
 static void release(casimir_request *r)
 {
-    give_pinned(r->plan->ctx, r);
+    give_pinned(r->ctx, r);
     if (r->done_ev) cudaEventDestroy(r->done_ev);
     delete r;
 }
@@ -2198,7 +2200,7 @@ static void release(casimir_request *r)
 int casimir_force(casimir_ticket r, int wait_ms, double F[3], double *err_est, casimir_stats *st)
 {
     if (!r) return fail(CASIMIR_EINVAL, "ticket is NULL");
-    casimir_ctx *c = r->plan->ctx;
+    casimir_ctx *c = r->ctx;   // the plan may be gone once the request has finished
     std::unique_lock<std::mutex> lk(c->mu);
     auto ready = [&] { return r->state >= 2; };
     if (wait_ms < 0) c->cv.wait(lk, ready);
@@ -2211,7 +2213,7 @@ int casimir_force(casimir_ticket r, int wait_ms, double F[3], double *err_est, c
         st->queue_ms = r->t_admit - r->t_submit;
         st->device_ms = r->t_done - r->t_admit;
         st->total_ms = r->t_done - r->t_submit;
-        st->cell_updates = r->plan->cells * (int64_t)r->plan->data.prob.n_steps;
+        st->cell_updates = r->cell_updates;
         st->kernel_launches = r->launches;
     }
     const std::string msg = r->msg;
@@ -2229,7 +2231,7 @@ int casimir_force(casimir_ticket r, int wait_ms, double F[3], double *err_est, c
 int casimir_cancel(casimir_ticket r)
 {
     if (!r) return fail(CASIMIR_EINVAL, "ticket is NULL");
-    casimir_ctx *c = r->plan->ctx;
+    casimir_ctx *c = r->ctx;   // the plan may be gone once the request has finished
     std::lock_guard<std::mutex> lk(c->mu);
     r->cancel = true;
     c->cv.notify_all();

@@ -153,7 +153,9 @@ struct casimir_plan {
 };
 
 struct casimir_request {
-    casimir_plan_t *plan = nullptr;
+    casimir_plan_t *plan = nullptr;   // until the request has finished
+    casimir_ctx *ctx = nullptr;
+    int64_t cell_updates = 0;         // of the whole run
     uint64_t tag = 0;
     std::atomic<int> state{0};   // 0 queued, 1 running, 2 done, 3 failed
     std::atomic<int> status{0};

@@ -1,0 +1,57 @@
+"""The engine's host side on the CPU: the library linked against a fake CUDA runtime (host_engine.py)."""
+import gc
+import os
+import subprocess
+import sys
+
+import pytest
+
+import host_engine
+import paper_0906_5170_gb300 as pk
+import workloads as W
+
+TESTS = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def lib_path():
+    return host_engine.build()
+
+
+@pytest.fixture
+def fake(lib_path):
+    old = pk.capi._lib
+    L = host_engine.load(lib_path)
+    L.fake_reset()
+    yield L
+    gc.collect()             # handles of the fake library are released by it
+    pk.capi._lib = old
+
+
+TICKET_AFTER_PLAN = """
+import ctypes, sys
+sys.path[:0] = [{root!r}, {tests!r}]
+import host_engine, workloads as W
+import paper_0906_5170_gb300 as pk
+L = host_engine.load({lib!r})
+c = pk.Context(0)
+for cancel in (False, True):
+    pl = c.plan(W.piston_small(n_steps=60, precision="fp32"))
+    updates = pl.info()["cell_updates"]
+    t = pl.submit()
+    pl.close()                     # returns once the request has finished
+    if cancel:
+        t.cancel()                 # of a finished request: no effect
+    F, err, st = t.force(-1)
+    assert st["cell_updates"] == updates, st
+c.close()
+"""
+
+
+def test_ticket_outlives_its_plan(lib_path):
+    # a plan has to live until its requests have finished, and its tickets are collected after that:
+    # casimir_force and casimir_cancel read nothing of the plan (freed memory is overwritten here)
+    script = TICKET_AFTER_PLAN.format(root=os.path.dirname(TESTS), tests=TESTS, lib=lib_path)
+    r = subprocess.run([sys.executable, "-c", script], env=dict(os.environ, MALLOC_PERTURB_="165"),
+                       capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, (r.returncode, r.stderr[-2000:])
