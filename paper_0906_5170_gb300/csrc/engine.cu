@@ -913,11 +913,12 @@ static int take_pinned(casimir_ctx *c, size_t need, casimir_request *r)
     return CASIMIR_OK;
 }
 
-// Leaves it to the next request, or frees it (a large one, or when enough are kept).
+// Leaves it to the next request, or frees it (a large one, when enough are kept, or one that copies may still
+// be in flight to: a request that failed before its results landed).
 static void give_pinned(casimir_ctx *c, casimir_request *r)
 {
     if (!r->h_acc) return;
-    if (r->h_bytes <= casimir_ctx::PINNED_MAX) {
+    if (r->landed && r->h_bytes <= casimir_ctx::PINNED_MAX) {
         std::lock_guard<std::mutex> lk(c->pinned_mu);
         for (auto &sp : c->pinned)
             if (!sp.first) {
@@ -1520,6 +1521,7 @@ static void finish_request(casimir_ctx *c, casimir_request *r, int status)
     dev_free(c, r->block);
     c->used -= align256(P->field_elems * P->rsize) + 2 * align256((ns + 1) * 8);
     r->block = nullptr;
+    r->landed = true;
     r->t_done = now_ms();
     if (status == CASIMIR_OK && *(const int *)(r->h_acc + 2 * ns)) {   // a resident cluster's wait ran out
         status = CASIMIR_ECUDA;

@@ -170,7 +170,7 @@ struct casimir_request {
     double *h_acc = nullptr;  // pinned copy-back (acc, tail, then the status word)
     size_t h_bytes = 0;
     cudaEvent_t done_ev = nullptr;
-    bool copy_issued = false;
+    bool copy_issued = false, landed = false;
     std::vector<double> per_sim;
     std::string msg;          // why the request failed (the worker's error message)
     // the request's simulations run in waves (contiguous ranges in plan order)

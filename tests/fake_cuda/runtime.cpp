@@ -18,9 +18,10 @@ std::mutex mu;
 std::map<const void *, std::string> names;   // registered kernels
 std::map<std::string, int64_t> counts;       // launches by kernel name
 std::vector<std::pair<std::string, double>> costs;
-int64_t queries = 0, captures = 0;
+int64_t queries = 0, captures = 0, host_frees = 0;
 double clock_ms = 0;
 int fail_resident = 0;                       // resident launches report a wait that ran out
+int fail_late = 0;                           // 1: copies back never land, and the stream fails from the first look at one on (2)
 bool capturing = false;
 std::vector<std::string> captured;
 thread_local int device = 0;
@@ -67,6 +68,8 @@ int64_t fake_launches(const char *part)
 int64_t fake_queries() { return queries; }
 int64_t fake_captures() { return captures; }
 void fake_cost(const char *part, double ms) { costs.insert(costs.begin(), {part, ms}); }
+int64_t fake_host_frees() { return host_frees; }
+void fake_fail_late(int on) { fail_late = on; }
 void fake_fail_resident(int on) { fail_resident = on; }
 int fake_device(int set)
 {
@@ -78,8 +81,8 @@ void fake_reset()
     std::lock_guard<std::mutex> lk(mu);
     counts.clear();
     costs.clear();
-    queries = captures = 0;
-    fail_resident = 0;
+    queries = captures = host_frees = 0;
+    fail_resident = fail_late = 0;
     clock_ms = 0;
 }
 
@@ -131,7 +134,11 @@ cudaError_t cudaMemGetInfo(size_t *f, size_t *t) { *f = *t = (size_t)4 << 30; re
 cudaError_t cudaMalloc(void **p, size_t n) { *p = calloc(1, n); return *p ? cudaSuccess : cudaErrorMemoryAllocation; }
 cudaError_t cudaFree(void *p) { free(p); return cudaSuccess; }
 cudaError_t cudaMallocHost(void **p, size_t n) { return cudaMalloc(p, n); }
-cudaError_t cudaFreeHost(void *p) { return cudaFree(p); }
+cudaError_t cudaFreeHost(void *p)
+{
+    ++host_frees;
+    return cudaFree(p);
+}
 cudaError_t cudaMemcpy(void *d, const void *s, size_t n, cudaMemcpyKind) { memcpy(d, s, n); return cudaSuccess; }
 cudaError_t cudaMemcpyAsync(void *d, const void *s, size_t n, cudaMemcpyKind, cudaStream_t) { memcpy(d, s, n); return cudaSuccess; }
 cudaError_t cudaMemsetAsync(void *d, int v, size_t n, cudaStream_t) { memset(d, v, n); return cudaSuccess; }
@@ -142,14 +149,18 @@ const char *cudaGetErrorString(cudaError_t) { return "error of the fake runtime"
 // ---- streams, events, graphs -----------------------------------------------------------
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) { *s = (cudaStream_t)malloc(1); return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { free(s); return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return fail_late == 2 ? cudaErrorLaunchFailure : cudaSuccess; }
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t *e) { *e = (cudaEvent_t) new Event; return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return cudaEventCreate(e); }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { delete (Event *)e; return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t) { ((Event *)e)->at = clock_ms; return cudaSuccess; }
 cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
-cudaError_t cudaEventQuery(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventQuery(cudaEvent_t)
+{
+    if (fail_late) fail_late = 2;
+    return fail_late ? cudaErrorNotReady : cudaSuccess;
+}
 cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t a, cudaEvent_t b)
 {
     *ms = (float)(((Event *)b)->at - ((Event *)a)->at);

@@ -31,7 +31,7 @@ def load(path):
         f = getattr(L, name)
         f.restype = res
         f.argtypes = args
-    for name in ("fake_launches", "fake_queries", "fake_captures"):
+    for name in ("fake_launches", "fake_queries", "fake_captures", "fake_host_frees"):
         getattr(L, name).restype = ctypes.c_int64
     L.fake_launches.argtypes = [ctypes.c_char_p]
     L.fake_cost.argtypes = [ctypes.c_char_p, ctypes.c_double]

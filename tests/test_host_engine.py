@@ -55,3 +55,19 @@ def test_ticket_outlives_its_plan(lib_path):
     r = subprocess.run([sys.executable, "-c", script], env=dict(os.environ, MALLOC_PERTURB_="165"),
                        capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, (r.returncode, r.stderr[-2000:])
+
+
+def test_result_buffer_of_a_failed_run_is_not_reused(fake):
+    # its copies may still be in flight: only a request whose results have landed leaves its pinned buffer
+    # to the next one
+    c = pk.Context(0)
+    pl = c.plan(W.piston_small(n_steps=60, precision="fp32"))
+    pl.run()
+    assert fake.fake_host_frees() == 0          # kept
+    fake.fake_fail_late(1)
+    with pytest.raises(pk.CasimirError):
+        pl.run()
+    fake.fake_fail_late(0)
+    assert fake.fake_host_frees() == 1
+    pl.run()
+    c.close()
