@@ -254,6 +254,9 @@ class Context:
         check(lib().casimir_ctx_create(int(device), int(hbm_budget_bytes), ctypes.byref(h)))
         self.h = h
         self._plans = weakref.WeakSet()
+        # their handles: what of them is still to be released (the garbage collector may finalise the context
+        # before a plan, and clears the weak references first)
+        self._handles = set()
         if stream is not None:
             check(lib().casimir_ctx_set_stream(self.h, ctypes.c_void_p(int(stream))))
 
@@ -288,6 +291,8 @@ class Context:
         if self.h:
             for p in list(self._plans):      # plans must be released before their context
                 p.close()
+            while self._handles:
+                lib().casimir_plan_destroy(self._handles.pop())
             lib().casimir_ctx_destroy(self.h)
             self.h = None
 
@@ -315,6 +320,7 @@ class Plan:
         self.h = h
         if ctx is not None:
             ctx._plans.add(self)
+            ctx._handles.add(h.value)
 
     def options(self):
         o = PlanOptions()
@@ -403,7 +409,10 @@ class Plan:
 
     def close(self):
         if self.h:
-            lib().casimir_plan_destroy(self.h)
+            if self.ctx is None or self.h.value in self.ctx._handles:
+                if self.ctx is not None:
+                    self.ctx._handles.discard(self.h.value)
+                lib().casimir_plan_destroy(self.h)
             self.h = None
 
     def __del__(self):

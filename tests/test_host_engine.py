@@ -71,3 +71,28 @@ def test_result_buffer_of_a_failed_run_is_not_reused(fake):
     assert fake.fake_host_frees() == 1
     pl.run()
     c.close()
+
+
+EXIT_WITH_OPEN_HANDLES = """
+import sys
+sys.path[:0] = [{root!r}, {tests!r}]
+import host_engine, workloads as W
+import paper_0906_5170_gb300 as pk
+L = host_engine.load({lib!r})
+c = pk.Context(0)
+pl = c.plan(W.piston_small(n_steps=60, precision="fp32"))
+t = pl.submit()
+t.force(-1)
+def hold():
+    return c, pl, t
+{end}
+"""
+
+
+@pytest.mark.parametrize("end", ["", "hold.cycle = [c, pl, hold]; del c, pl, t, hold; import gc; gc.collect()"])
+def test_context_and_plans_are_released_in_any_order(lib_path, end):
+    # the garbage collector finalises a context and its plans in no set order, weak references cleared first
+    script = EXIT_WITH_OPEN_HANDLES.format(root=os.path.dirname(TESTS), tests=TESTS, lib=lib_path, end=end)
+    r = subprocess.run([sys.executable, "-c", script], env=dict(os.environ, MALLOC_PERTURB_="165"),
+                       capture_output=True, text=True, timeout=120)
+    assert r.returncode == 0, (r.returncode, r.stderr[-2000:])
