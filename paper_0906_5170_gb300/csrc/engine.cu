@@ -304,6 +304,40 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
     return q->smem <= RES_SMEM_MAX;
 }
 
+// The caller's current device, made so again at the end of a scope.
+struct DeviceScope {
+    int before = -1;
+    explicit DeviceScope(int device)
+    {
+        if (cudaGetDevice(&before) != cudaSuccess || before == device || cudaSetDevice(device) != cudaSuccess) before = -1;
+    }
+    ~DeviceScope()
+    {
+        if (before >= 0) cudaSetDevice(before);
+    }
+};
+
+// 2D TM/TE and cylindrical plans on a device: the first shape of the resident march that holds them.
+static void choose_resident(casimir_plan_t *P)
+{
+    const PlanData &D = P->data;
+    const bool cyl = !D.sims.empty() && D.geos[D.sims[0].geo].cyl;
+    if (!P->ctx || D.sims.empty() || (!cyl && D.geos[D.sims[0].geo].family == FAM_FULL) ||
+        12 * (int64_t)D.prob.n[0] * D.prob.n[1] >= ((int64_t)1 << 31)) return;
+    DeviceScope dev(P->ctx->device);
+    for (Res2dShape &q : res2d_shapes(cyl, P->fp64, D.prob.n[0], D.prob.n[1], (int)D.sims.size()))
+        if (resident_tables(P, &q)) {
+            P->resident = true;
+            P->res = q;
+            return;
+        }
+    P->resW.clear();
+    P->resC.clear();
+    P->resE.clear();
+    P->resT.clear();
+    P->resNT.clear();
+}
+
 // allow_resident: the caller left steps_per_launch to the default
 static int prepare_plan(casimir_plan_t *P, bool allow_resident)
 {
@@ -359,24 +393,7 @@ static int prepare_plan(casimir_plan_t *P, bool allow_resident)
             }
         P->pml_off.push_back(po);
     }
-    // 2D TM/TE and cylindrical plans on a device: the first shape of the resident march that holds them
-    const bool cyl = !D.sims.empty() && D.geos[D.sims[0].geo].cyl;
-    if (allow_resident && P->ctx && !D.sims.empty() && (cyl || D.geos[D.sims[0].geo].family != FAM_FULL) &&
-        12 * (int64_t)D.prob.n[0] * D.prob.n[1] < ((int64_t)1 << 31)) {
-        cudaSetDevice(P->ctx->device);
-        for (Res2dShape &q : res2d_shapes(cyl, P->fp64, D.prob.n[0], D.prob.n[1], (int)D.sims.size()))
-            if (resident_tables(P, &q)) {
-                P->resident = true;
-                P->res = q;
-                break;
-            }
-        if (!P->resident) {
-            P->resW.clear();
-            P->resC.clear();
-            P->resE.clear();
-            P->resT.clear();
-        }
-    }
+    if (allow_resident) choose_resident(P);
     // sims, tiles, entries, sources
     int64_t off = 0;
     std::map<int, std::vector<int>> march_variants;   // per geometry: kernel variant of each march tile

@@ -96,3 +96,13 @@ def test_context_and_plans_are_released_in_any_order(lib_path, end):
     r = subprocess.run([sys.executable, "-c", script], env=dict(os.environ, MALLOC_PERTURB_="165"),
                        capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, (r.returncode, r.stderr[-2000:])
+
+
+def test_planning_leaves_the_callers_device_current(fake):
+    c = pk.Context(1)
+    fake.fake_device(0)
+    for p in (W.piston_small(n_steps=60, precision="fp32"), W.cylinder_piston(10, [0, 1], t_max=2.0)):
+        with_resident = c.plan(p)
+        assert fake.fake_device(-1) == 0
+        with_resident.close()
+    c.close()
