@@ -325,7 +325,8 @@ static void choose_resident(casimir_plan_t *P)
     if (!P->ctx || D.sims.empty() || (!cyl && D.geos[D.sims[0].geo].family == FAM_FULL) ||
         12 * (int64_t)D.prob.n[0] * D.prob.n[1] >= ((int64_t)1 << 31)) return;
     DeviceScope dev(P->ctx->device);
-    for (Res2dShape &q : res2d_shapes(cyl, P->fp64, D.prob.n[0], D.prob.n[1], (int)D.sims.size()))
+    ResShapes shapes(cyl, P->fp64, D.prob.n[0], D.prob.n[1], (int)D.sims.size());
+    for (Res2dShape q; shapes.next(&q);)
         if (resident_tables(P, &q)) {
             P->resident = true;
             P->res = q;

@@ -253,7 +253,24 @@ constexpr int RES_LAUNCH_STEPS = 192;         // time steps of one launch at mos
 constexpr int RES_LAUNCH_INDICES = RES_LAUNCH_STEPS / 3;
 cudaError_t res2d_prepare();
 int res2d_proj_bytes(const Res2dShape &q);      // shared memory of the projection's history and sums
-std::vector<Res2dShape> res2d_shapes(int cyl, int fp64, int nx, int ny, int nsims);
+// The shapes of the resident march that hold an nx x ny simulation on the current device, the fastest by the
+// model first.  How many clusters of a shape fit the device is asked (a driver call) only for shapes that can
+// still be the next one.
+class ResShapes {
+public:
+    ResShapes(int cyl, int fp64, int nx, int ny, int nsims);
+    bool next(Res2dShape *q, double *clocks = nullptr);   // false: no more
+
+private:
+    struct Shape {
+        double t;       // the model's clocks of a step: at least (exact: just) this
+        int order;
+        bool exact;
+        Res2dShape q;
+    };
+    int nsims, sms = 1;
+    std::vector<Shape> heap;
+};
 // launch indices launch .. launch + count - 1
 void launch_res2d(const Res2dShape &q, const void *sims, int nsims, int64_t launch, int count, cudaStream_t st);
 

@@ -705,8 +705,7 @@ static int clusters_resident(const void *k, const Res2dShape &q, bool alone)
     return fit;
 }
 
-// Shapes that hold an nx x ny simulation, the fastest by the model first.  The model's clocks of a step
-// for the warps that share an SM: FP32 the larger of 137 a warp (measured with 16 warps; about 300
+// The model's clocks of a step, `share` CTAs to an SM, for the warps that share it: FP32 the larger of 137 a warp (measured with 16 warps; about 300
 // instructions a warp, 45% of the issue slots) and of one warp's own chain (1200; 1750 when rows come from other CTAs);
 // FP64 its arithmetic at two lanes a clock and SM times 1.22, plus 700.  Simulations beyond those resident
 // at once run one after the other.  Measured in FP32 (Gcell-updates/s, 400 x 166 cells, 640 simulations,
@@ -717,14 +716,29 @@ static int clusters_resident(const void *k, const Res2dShape &q, bool alone)
 // idle, ran at 436 : 409 (FP32, 400 x 200, 320 simulations) and 30.1 : 28.5 (FP64, 256 x 200, 160).  Cylindrical, FP32: 27.5 clocks a
 // warp and cell of a thread (29 with three rows, which spill a little) and 770, at least 2300; 126 simulations of
 // 60 x 400: two rows in clusters of 6 229 Gcell-updates/s, of 7 177, of 9 202, three rows in clusters of 5 220, of 6 224.
-std::vector<Res2dShape> res2d_shapes(int cyl, int fp64, int nx, int ny, int nsims)
+static double step_clocks(const Res2dShape &q, int share)
 {
-    std::vector<std::pair<double, Res2dShape>> found;
+    const int cx = q.fp64 ? 2 : 4;
+    const double warps = share * (q.threads / 32);
+    if (q.cyl) return q.fp64 ? 1.22 * warps * 16.0 * q.rb * cx * 40.0 + 1000.0 : std::max(2300.0, warps * q.rb * cx * (q.rb == 3 ? 29.0 : 27.5) + 770.0);
+    if (q.fp64) return 1.22 * warps * 16.0 * q.rb * cx * 9.0 + 700.0;
+    const double chain = q.cluster > 1 ? 1750.0 : 1200.0, issue = (q.rb == 4 ? 137.0 : 120.0) * warps;
+    return std::max(chain, issue) + 0.1 * std::min(chain, issue);
+}
+
+static bool later(double t, int order, double t2, int order2) { return t != t2 ? t > t2 : order > order2; }
+
+ResShapes::ResShapes(int cyl, int fp64, int nx, int ny, int nsims_) : nsims(nsims_)
+{
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        return;
+    }
     const int cx = fp64 ? 2 : 4;
     const int tcols = (nx + cx - 1) / cx;
     for (int rb : {1, 2, 3, 4}) {
-        const void *k = res_kernel(cyl, fp64, rb);
-        if (!k) continue;
+        if (!res_kernel(cyl, fp64, rb)) continue;
         const int nb = (ny + rb - 1) / rb;                       // bands of rb or rb - 1 rows
         if (rb > 1 && ny / nb < rb - 1) continue;
         for (int c = 1; c <= RES_CLUSTER_MAX && c <= nb; ++c) {
@@ -741,27 +755,49 @@ std::vector<Res2dShape> res2d_shapes(int cyl, int fp64, int nx, int ny, int nsim
             int cw = 0;
             q.smem = (threads * res_words(cyl, fp64, rb, &cw) + (cyl ? RES_RAD * tcols : 0)) * 16 + RES_LAUNCH_STEPS * 8;   // (cyl: radial factors)
             if (q.smem > RES_SMEM_MAX) continue;
-            const int fit1 = clusters_resident(k, q, true), fit = std::max(fit1, clusters_resident(k, q, false));
-            if (fit1 < 1) continue;
-            const int share = std::max(1, std::min((nsims + fit1 - 1) / fit1, fit / fit1));   // CTAs on an SM
-            const int waves = (nsims + fit1 * share - 1) / (fit1 * share);
-            const double warps = share * (threads / 32);
-            double t;
-            if (cyl) {
-                t = fp64 ? 1.22 * warps * 16.0 * rb * cx * 40.0 + 1000.0 : std::max(2300.0, warps * rb * cx * (rb == 3 ? 29.0 : 27.5) + 770.0);
-            } else if (fp64) {
-                t = 1.22 * warps * 16.0 * rb * cx * 9.0 + 700.0;
-            } else {
-                const double chain = c > 1 ? 1750.0 : 1200.0, issue = (rb == 4 ? 137.0 : 120.0) * warps;
-                t = std::max(chain, issue) + 0.1 * std::min(chain, issue);
+            // With `share` CTAs to an SM no more clusters run at once than the SMs hold so many times, nor than the
+            // SMs' shared memory (228 KB, 1 KB of it a CTA's own) and threads allow.
+            const int alone = std::max(1, sms / c);
+            const int most = std::max(alone, sms * std::min(228 * 1024 / (q.smem + 1024), 2048 / threads) / c);
+            double t = 0;
+            for (int share = 1; share == 1 || (share - 1) * alone < std::min(most, nsims); ++share) {
+                const int at_once = std::min(most, alone * share);
+                const double ts = (nsims + at_once - 1) / at_once * step_clocks(q, share);
+                if (share == 1 || ts < t) t = ts;
             }
-            found.push_back({waves * t, q});
+            heap.push_back({t, (int)heap.size(), false, q});
         }
     }
-    std::stable_sort(found.begin(), found.end(), [](const auto &x, const auto &y) { return x.first < y.first; });
-    std::vector<Res2dShape> out;
-    for (auto &f : found) out.push_back(f.second);
-    return out;
+    std::make_heap(heap.begin(), heap.end(), [](const Shape &x, const Shape &y) { return later(x.t, x.order, y.t, y.order); });
+}
+
+bool ResShapes::next(Res2dShape *q, double *clocks)
+{
+    const auto cmp = [](const Shape &x, const Shape &y) { return later(x.t, x.order, y.t, y.order); };
+    while (!heap.empty()) {
+        std::pop_heap(heap.begin(), heap.end(), cmp);
+        Shape &s = heap.back();
+        if (s.exact) {
+            *q = s.q;
+            if (clocks) *clocks = s.t;
+            heap.pop_back();
+            return true;
+        }
+        const void *k = res_kernel(s.q.cyl, s.q.fp64, s.q.rb);
+        const int fit1 = clusters_resident(k, s.q, true);
+        // CTAs on an SM: one if each simulation's cluster finds SMs of its own
+        const int fit = nsims > fit1 ? std::max(fit1, clusters_resident(k, s.q, false)) : fit1;
+        if (fit1 < 1) {
+            heap.pop_back();
+            continue;
+        }
+        const int share = std::max(1, std::min((nsims + fit1 - 1) / fit1, fit / fit1));
+        const int waves = (nsims + fit1 * share - 1) / (fit1 * share);
+        s.t = waves * step_clocks(s.q, share);
+        s.exact = true;
+        std::push_heap(heap.begin(), heap.end(), cmp);
+    }
+    return false;
 }
 
 }  // namespace cas

@@ -71,6 +71,15 @@ void fake_cost(const char *part, double ms) { costs.insert(costs.begin(), {part,
 int64_t fake_host_frees() { return host_frees; }
 void fake_fail_late(int on) { fail_late = on; }
 void fake_fail_resident(int on) { fail_resident = on; }
+// The first `most` shapes of the resident march and the model's clocks for each, in the order they come.
+int fake_res_shapes(int cyl, int fp64, int nx, int ny, int nsims, int most, int *rows_cluster, double *clocks)
+{
+    cas::ResShapes shapes(cyl, fp64, nx, ny, nsims);
+    cas::Res2dShape q;
+    int n = 0;
+    while (n < most && shapes.next(&q, &clocks[n])) rows_cluster[n++] = 100 * q.rb + q.cluster;
+    return n;
+}
 int fake_device(int set)
 {
     if (set >= 0) device = set;

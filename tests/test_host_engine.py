@@ -1,4 +1,5 @@
 """The engine's host side on the CPU: the library linked against a fake CUDA runtime (host_engine.py)."""
+import ctypes
 import gc
 import os
 import subprocess
@@ -106,3 +107,22 @@ def test_planning_leaves_the_callers_device_current(fake):
         assert fake.fake_device(-1) == 0
         with_resident.close()
     c.close()
+
+
+SHAPE_SIZES = [(60, 20, 96), (3, 12, 4), (400, 166, 640), (400, 80, 64), (512, 512, 64), (128, 128, 320), (37, 901, 7), (251, 93, 40)]
+
+
+@pytest.mark.parametrize("cyl,fp64", [(0, 0), (0, 1), (1, 0), (1, 1)])
+@pytest.mark.parametrize("nx,ny,nsims", SHAPE_SIZES)
+def test_resident_shapes_come_best_first_and_are_looked_up_as_needed(fake, cyl, fp64, nx, ny, nsims):
+    # the order is that of the model over every shape that fits, ties in the order of rows and cluster size
+    def first(most):
+        shapes, clocks = (ctypes.c_int * 64)(), (ctypes.c_double * 64)()
+        n = fake.fake_res_shapes(cyl, fp64, nx, ny, nsims, most, shapes, clocks)
+        return [(clocks[i], shapes[i]) for i in range(n)]
+    every = first(64)
+    assert every == sorted(every) and len(set(every)) == len(every)
+    queries = fake.fake_queries()
+    fake.fake_reset()
+    assert first(1) == every[:1]
+    assert fake.fake_queries() <= max(4, 2 * queries // 3)
