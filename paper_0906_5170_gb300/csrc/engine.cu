@@ -1513,7 +1513,8 @@ static int run_chunk(casimir_ctx *c, int k)
         if (c->groups[gi].ntiles > 0)
             per_step += ((gi >= 2 && gi < 10) || (gi >= casimir_ctx::G_LINE3 && gi < casimir_ctx::G_CYL)) ? 2 : 1;
     const int64_t res_launches = (int64_t)c->nres * ((k + RES_LAUNCH_INDICES - 1) / RES_LAUNCH_INDICES);
-    for (casimir_request *r : c->active) r->launches += (int64_t)k * per_step + res_launches + (steps ? (k + GRAPH_INDICES - 1) / GRAPH_INDICES : 0);
+    const int64_t bumps = !steps ? 0 : no_graphs ? 1 : k / GRAPH_INDICES + k % GRAPH_INDICES;   // one per graph replayed
+    for (casimir_request *r : c->active) r->launches += (int64_t)k * per_step + res_launches + bumps;
     return CASIMIR_OK;
 }
 

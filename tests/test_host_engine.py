@@ -126,3 +126,13 @@ def test_resident_shapes_come_best_first_and_are_looked_up_as_needed(fake, cyl, 
     fake.fake_reset()
     assert first(1) == every[:1]
     assert fake.fake_queries() <= max(4, 2 * queries // 3)
+
+
+@pytest.mark.parametrize("steps,per_launch", [(90, 3), (301, 3), (64, 1), (77, 2)])
+def test_kernel_launches_are_counted(fake, steps, per_launch):
+    c = pk.Context(0)
+    pl = c.plan(W.piston_small(n_steps=steps, precision="fp32"), options={"steps_per_launch": per_launch})
+    fake.fake_reset()
+    st = pl.run()[2]
+    assert st["kernel_launches"] == fake.fake_launches(b"") - fake.fake_launches(b"inject")
+    c.close()
