@@ -1572,15 +1572,11 @@ static int engine_iterate(casimir_ctx *c)
             if (only_resident(c)) {
                 // short launches go several to a chunk (about 2 ms, between which the host looks at the queue)
                 if (c->index_ms > 0) k = (int)std::min<int64_t>(rem, std::max(64.0, std::min(1024.0, 2.0 / c->index_ms)));
-                // the watchdog is checked between chunks: these are cut to about a thousandth of its limit (a
-                // power of two indices)
+                // the watchdog is checked between chunks: these are cut to a twentieth of its limit.  (A chunk loads
+                // and stores the fields, and the host waits for it: about 60 us; cut to a thousandth of a limit of
+                // 200 ms, a run of 53 ms took 96.)
                 const double wd = c->watchdog_ms.load();
-                if (wd > 0) {
-                    int cut = 8;
-                    if (c->index_ms > 0)
-                        for (cut = 1; cut < k && 2 * cut * c->index_ms <= 1e-3 * wd;) cut *= 2;
-                    k = std::min(k, cut);
-                }
+                if (wd > 0) k = c->index_ms > 0 ? (int)std::max(1.0, std::min<double>(k, 0.05 * wd / c->index_ms)) : std::min(k, 8);
             }
             int rc = run_chunk(c, k);
             if (rc) return rc;

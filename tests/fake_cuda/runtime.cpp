@@ -1,6 +1,6 @@
 // A CUDA runtime without a GPU, for tests of the engine's host side: device memory is host memory, kernels
 // do not run but are counted by name, graphs replay what was launched while they were captured, and the
-// event clock advances by a settable time per kernel launch.
+// event clock advances by a settable time per kernel launch (resident marches: per launch of the most indices).
 #include <cuda_runtime.h>
 
 #include <cstdlib>
@@ -29,7 +29,7 @@ thread_local int device = 0;
 struct Event { double at = 0; };
 struct Graph { std::vector<std::string> kernels; };
 
-void run(const std::string &k)
+void run(const std::string &k, double part = 1)
 {
     if (capturing) {
         captured.push_back(k);
@@ -38,17 +38,17 @@ void run(const std::string &k)
     ++counts[k];
     for (const auto &c : costs)
         if (k.find(c.first) != std::string::npos) {
-            clock_ms += c.second;
+            clock_ms += part * c.second;
             break;
         }
 }
 
-cudaError_t launch(const void *f)
+cudaError_t launch(const void *f, double part = 1)
 {
     std::lock_guard<std::mutex> lk(mu);
     auto it = names.find(f);
     if (it == names.end()) return cudaErrorInvalidDeviceFunction;
-    run(it->second);
+    run(it->second, part);
     return cudaSuccess;
 }
 
@@ -122,7 +122,7 @@ cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void **, size_t, cuda
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *, const void *f, void **args)
 {
     if (fail_resident) *(*(const cas::DevRes *const *)args[0])->status = 1;
-    return launch(f);
+    return launch(f, *(const int *)args[2] / (double)cas::RES_LAUNCH_INDICES);
 }
 cudaError_t cudaFuncSetAttribute(const void *, cudaFuncAttribute, int) { return cudaSuccess; }
 // clusters that fit 152 SMs of 228 KB shared memory and 64 K registers (128 a thread), in one pool

@@ -136,3 +136,21 @@ def test_kernel_launches_are_counted(fake, steps, per_launch):
     st = pl.run()[2]
     assert st["kernel_launches"] == fake.fake_launches(b"") - fake.fake_launches(b"inject")
     c.close()
+
+
+@pytest.mark.parametrize("limit_ms", [50.0, 200.0, 1000.0])
+def test_a_watched_run_takes_few_more_launches(fake, limit_ms):
+    # 64 simulations of 400 x 80: 0.5 ms a launch of 192 steps; a watched chunk still ends well inside the limit
+    p = W.config2_piston(W.config2_heights()[0], n_harm=4, n_steps=20000)
+    c = pk.Context(0)
+    pl = c.plan(p)
+    fake.fake_reset()
+    fake.fake_cost(b"k_res2d", 0.5)
+    pl.run()
+    plain = fake.fake_launches(b"k_res2d")
+    c.set_watchdog(limit_ms)
+    fake.fake_reset()
+    fake.fake_cost(b"k_res2d", 0.5)
+    pl.run()
+    assert plain <= fake.fake_launches(b"k_res2d") <= 1.05 * plain + 2
+    c.close()
