@@ -71,22 +71,22 @@ __device__ __forceinline__ bool mb_try(unsigned mb, unsigned parity)
                  : "memory");
     return ok;
 }
-// Waits for the phase of the given parity; gives up after a second, which no correct run comes near, so
-// that the kernel always ends.
+// Tries of a wait before it gives up, so that the kernel always ends.  A try that finds the phase unfinished
+// takes 3.8 us (the hardware's limit on its suspension), all of them half a second of the kernel's own time,
+// which no correct run comes near; no clock is read, so time the context is switched away does not count.
+#ifndef RES_WAIT_TRIES
+#define RES_WAIT_TRIES (1 << 17)
+#endif
 __device__ __noinline__ bool mb_wait_long(unsigned mb, unsigned parity)
 {
-    unsigned long long t0, t1;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
-    for (int i = 0; i < 1 << 26; ++i) {
+    for (int i = 64; i < RES_WAIT_TRIES; ++i)
         if (mb_try(mb, parity)) return true;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
-        if (t1 - t0 > 1000000000ull) break;
-    }
     return false;
 }
+// Waits for the phase of the given parity; false: it gave up.
 __device__ __forceinline__ bool mb_wait(unsigned mb, unsigned parity)
 {
-    for (int i = 0; i < 64; ++i)
+    for (int i = 0; i < (RES_WAIT_TRIES < 64 ? RES_WAIT_TRIES : 64); ++i)
         if (mb_try(mb, parity)) return true;
     return mb_wait_long(mb, parity);
 }
