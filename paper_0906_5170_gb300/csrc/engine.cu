@@ -819,7 +819,7 @@ static int prepare_plan(casimir_plan_t *P, bool allow_resident)
                                align256(P->lorc_all.size() * P->rsize) + align256(P->resW.size() * sizeof(DevResWarp)) +
                                align256(P->resC.size() * sizeof(DevResCta)) + align256(P->resE.size() * sizeof(DevEntR)) +
                                align256(P->resT.size() * sizeof(short)));
-    P->request_bytes = (int64_t)(align256(P->field_elems * P->rsize) + 2 * align256((P->sims.size() + 1) * 8) +
+    P->request_bytes = (int64_t)(align256(P->field_elems * P->rsize) + 2 * align256(P->sims.size() * 8) +
                                  P->tiles.size() * sizeof(DevTile) + P->tiles6.size() * sizeof(DevTile6) +
                                  P->tiles2.size() * sizeof(DevTile2) + P->tilesM.size() * sizeof(DevTile) +
                                  P->sims.size() * std::max(sizeof(DevResCyl), sizeof(DevSim6)));
@@ -954,7 +954,7 @@ static int admit(casimir_ctx *c, casimir_request *r)
     casimir_plan_t *P = r->plan;
     int rc = upload_plan(P, c->stream);
     if (rc) return rc;
-    size_t bf = align256(P->field_elems * P->rsize), ba = align256((P->sims.size() + 1) * 8);   // tail sums, then a status word
+    size_t bf = align256(P->field_elems * P->rsize), ba = align256(P->sims.size() * 8);
     void *blk;
     rc = dev_alloc(c, bf + 2 * ba, &blk);
     if (rc) return rc;
@@ -971,6 +971,7 @@ static int admit(casimir_ctx *c, casimir_request *r)
         rc = take_pinned(c, (2 * P->sims.size() + 1) * 8, r);
         if (rc) return rc;
     }
+    *r->status_word() = 0;
     // waves of consecutive simulations whose field blocks fit the wave budget
     r->waves.clear();
     r->waves_done = 0;
@@ -1162,7 +1163,7 @@ static int rebuild(casimir_ctx *c)
                     d.warps = P->dev.resw + hs.resw0;
                     d.ctas = P->dev.resc + hs.resc0;
                     d.ents = P->dev.rese + hs.rese0;
-                    d.status = (int *)(r->tail + P->sims.size());
+                    d.status = r->status_word();
                     d.gen_words = q.gen_words;
                     d.stage_words = q.stage_words;
                     d.ne_max = q.ne_max;
@@ -1538,11 +1539,11 @@ static void finish_request(casimir_ctx *c, casimir_request *r, int status)
     r->F[D.prob.force_axis] = s;
     r->err = te;
     dev_free(c, r->block);
-    c->used -= align256(P->field_elems * P->rsize) + 2 * align256((ns + 1) * 8);
+    c->used -= align256(P->field_elems * P->rsize) + 2 * align256(ns * 8);
     r->block = nullptr;
     r->landed = true;
     r->t_done = now_ms();
-    if (status == CASIMIR_OK && *(const int *)(r->h_acc + 2 * ns)) {   // a resident cluster's wait ran out
+    if (*r->status_word() && (status == CASIMIR_OK || status == CASIMIR_ECUDA)) {
         status = CASIMIR_ECUDA;
         r->msg = "resident march: a wait between the CTAs of a cluster ran out";
     }
@@ -1617,15 +1618,16 @@ static int engine_iterate(casimir_ctx *c)
         bool done = r->waves_done == r->waves.size();
         const double wd = c->watchdog_ms.load();
         bool timed_out = wd > 0 && now_ms() - r->t_admit > wd;
-        if (done || timed_out || r->cancel) {
+        const bool failed = *r->status_word() != 0;   // in the last chunk, which has ended
+        if (done || timed_out || r->cancel || failed) {
             if (!done) drop_waves(c, r);
             size_t ns = r->plan->sims.size();
             CUDA_TRY(cudaMemcpyAsync(r->h_acc, r->acc, ns * 8, cudaMemcpyDeviceToHost, c->stream));
-            CUDA_TRY(cudaMemcpyAsync(r->h_acc + ns, r->tail, (ns + 1) * 8, cudaMemcpyDeviceToHost, c->stream));
+            CUDA_TRY(cudaMemcpyAsync(r->h_acc + ns, r->tail, ns * 8, cudaMemcpyDeviceToHost, c->stream));
             if (!r->done_ev) CUDA_TRY(cudaEventCreateWithFlags(&r->done_ev, cudaEventDisableTiming));
             CUDA_TRY(cudaEventRecord(r->done_ev, c->stream));
             r->copy_issued = true;
-            if (!done) r->status = r->cancel ? CASIMIR_ECANCELED : CASIMIR_ETIMEOUT;
+            if (!done) r->status = r->cancel ? CASIMIR_ECANCELED : failed ? CASIMIR_ECUDA : CASIMIR_ETIMEOUT;
         }
     }
     {
@@ -2297,7 +2299,7 @@ int casimir_run(casimir_plan_t *P, double F[3], double *per_sim, casimir_stats *
     }
     give_pinned(c, &r);
     if (r.done_ev) cudaEventDestroy(r.done_ev);
-    if (status != CASIMIR_OK && rc == CASIMIR_OK) return fail(status, "run stopped");
+    if (status != CASIMIR_OK && rc == CASIMIR_OK) return fail(status, r.msg.empty() ? "run stopped" : r.msg);
     return status;
 }
 

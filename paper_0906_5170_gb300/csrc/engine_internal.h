@@ -167,8 +167,9 @@ struct casimir_request {
     int64_t launches = 0;
     void *block = nullptr;   // fields, acc, tail
     double *acc = nullptr, *tail = nullptr;
-    double *h_acc = nullptr;  // pinned copy-back (acc, tail, then the status word)
+    double *h_acc = nullptr;  // pinned copy-back (acc, tail), then a status word that resident kernels write themselves
     size_t h_bytes = 0;
+    volatile int *status_word() const { return (volatile int *)(h_acc + 2 * plan->sims.size()); }   // not 0: a wait ran out
     cudaEvent_t done_ev = nullptr;
     bool copy_issued = false, landed = false;
     std::vector<double> per_sim;

@@ -217,7 +217,7 @@ struct DevRes {
     const DevResWarp *warps;   // [cluster rank][warp]
     const DevResCta *ctas;     // [cluster rank]
     const DevEntR *ents;
-    int *status;               // set when a wait ran out
+    volatile int *status;      // set when a wait ran out (pinned host memory)
     const short *tile_pieces;  // [ntile + 1] pieces of each tile
     int64_t term_off;          // the launch's terms by piece and step, in doubles from s.fields
     int tcols, nb, k;          // threads per row band, row bands, time steps per launch index

@@ -154,3 +154,19 @@ def test_a_watched_run_takes_few_more_launches(fake, limit_ms):
     pl.run()
     assert plain <= fake.fake_launches(b"k_res2d") <= 1.05 * plain + 2
     c.close()
+
+
+@pytest.mark.parametrize("how", ["run", "submit"])
+def test_a_failed_resident_run_stops_at_its_chunk(fake, how):
+    # a wait that ran out is seen after the chunk it happened in, not at the end of the run's 20000 steps
+    c = pk.Context(0)
+    pl = c.plan(W.config2_piston(W.config2_heights()[0], n_harm=4, n_steps=20000))
+    fake.fake_reset()
+    fake.fake_fail_resident(1)
+    with pytest.raises(pk.CasimirError) as e:
+        pl.run() if how == "run" else pl.submit().force(-1)
+    assert e.value.code == pk.capi.ECUDA and "ran out" in str(e.value)
+    assert fake.fake_launches(b"k_res2d") == 1
+    fake.fake_fail_resident(0)
+    pl.run()                    # the next run's status is its own
+    c.close()
