@@ -91,6 +91,13 @@ __device__ __forceinline__ bool mb_wait(unsigned mb, unsigned parity)
     return mb_wait_long(mb, parity);
 }
 
+// The end of a thread whose wait ran out: its CTA's shared memory stays a while (about a millisecond; a copy
+// takes microseconds) for rows its neighbours sent that may still be in flight.
+__device__ __noinline__ void linger()
+{
+    for (int i = 0; i < 1000; ++i) __nanosleep(1000);
+}
+
 // bits of the packed per-thread state
 constexpr unsigned F_ACTIVE = 1u, F_SHORT = 2u, F_FARU = 4u, F_FARD = 8u, F_NEEDU = 16u, F_NEEDD = 32u, F_LEADU = 64u, F_LEADD = 128u,
                    F_LATE = 256u, F_STAGE = 512u, F_MINE = 1024u, F_DEAD = 2048u, F_FIRST = 4096u, F_STAGEW = 8192u;
