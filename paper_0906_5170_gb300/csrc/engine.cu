@@ -89,11 +89,7 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
 {
     const PlanData &D = P->data;
     const int cx = q->fp64 ? 2 : 4, nwarp = q->threads / 32, nx = D.prob.n[0], ny = D.prob.n[1];
-    P->resW.clear();
-    P->resC.clear();
-    P->resE.clear();
-    P->resT.clear();
-    P->resNT.clear();
+    P->clear_resident();
     q->stage_words = q->ne_max = q->np_max = q->npiece_max = q->ntile_max = 0;
     const int txk = q->cyl ? MARCH_W2 : tile_xk(P->opts.steps_per_launch == 3 ? 3 : 2), tx = (nx + txk - 1) / txk;   // tiles of the multi-step kernels
     const int tyk = q->cyl ? P->opts.march_rows : TILE_Y;
@@ -158,42 +154,48 @@ static bool resident_tables(casimir_plan_t *P, Res2dShape *q)
     };
     std::vector<DevResWarp> rec((size_t)q->cluster * nwarp);
     // The harmonics of a face share their sites: a simulation measured at the sites of an earlier one of its
-    // lattice, face and source component takes that one's tables with its own weights.
+    // lattice, face and source component takes that one's tables (resAt) with its own weights.
     struct Like {
         size_t sim;                   // the earlier simulation
-        int64_t e0;                   // its first entry
-        std::vector<Entry> meas;
+        const std::vector<Entry> *meas;
         std::vector<int> from;        // entry -> place in meas
     };
     std::map<std::array<int, 4>, Like> like;
+    std::deque<std::vector<Entry>> kept;   // cylindrical: the entries of the source's real set alone (prepare_plan)
+    size_t nmeas = 0;
+    for (const Sim &sm : D.sims) nmeas += sm.meas.size();
+    P->resE.reserve(nmeas);
     for (size_t si = 0; si < D.sims.size(); ++si) {
         const Sim &sm = D.sims[si];
-        std::fill(rec.begin(), rec.end(), DevResWarp{});
         const int arrays = q->cyl ? 3 : (sm.second_u ? 1 : 2);
-        // the sigma group's first array; cylindrical: the entries of the source's real set alone (prepare_plan)
-        const int arr0 = q->cyl ? 3 * sm.kind : (sm.second_u ? 0 : 1);
-        auto in_a = [](int arr) { return arr == 0 || arr == 1 || arr == 5; };
-        std::vector<Entry> meas;
-        for (const Entry &e : sm.meas)
-            if (!q->cyl || sm.src.empty() || in_a(e.arr) == in_a(sm.src[0].arr)) meas.push_back(e);
+        const int arr0 = q->cyl ? 3 * sm.kind : (sm.second_u ? 0 : 1);   // the sigma group's first array
+        const std::vector<Entry> *list = &sm.meas;
+        if (q->cyl && !sm.src.empty()) {
+            auto in_a = [](int arr) { return arr == 0 || arr == 1 || arr == 5; };
+            kept.emplace_back();
+            for (const Entry &e : sm.meas)
+                if (in_a(e.arr) == in_a(sm.src[0].arr)) kept.back().push_back(e);
+            list = &kept.back();
+        }
+        const std::vector<Entry> &meas = *list;
+        P->resE0.push_back((int64_t)P->resE.size());
         const std::array<int, 4> key{sm.geo, sm.face, sm.kind, sm.comp};
         auto lk = like.find(key);
-        if (lk != like.end() && D.sims[lk->second.sim].second_u == sm.second_u && lk->second.meas.size() == meas.size() &&
-            std::equal(meas.begin(), meas.end(), lk->second.meas.begin(), [](const Entry &x, const Entry &y) { return x.arr == y.arr && x.idx == y.idx; })) {
+        if (lk != like.end() && D.sims[lk->second.sim].second_u == sm.second_u && lk->second.meas->size() == meas.size() &&
+            std::equal(meas.begin(), meas.end(), lk->second.meas->begin(), [](const Entry &x, const Entry &y) { return x.arr == y.arr && x.idx == y.idx; })) {
             const Like &l = lk->second;
-            const size_t nw = rec.size(), nc = (size_t)q->cluster;
-            for (size_t v = 0; v < nw; ++v) P->resW.push_back(P->resW[l.sim * nw + v]);
-            for (size_t v = 0; v < nc; ++v) P->resC.push_back(P->resC[l.sim * nc + v]);
-            for (size_t v = 0; v <= RES_TILES; ++v) P->resT.push_back(P->resT[l.sim * (RES_TILES + 1) + v]);
-            P->resNT.push_back(P->resNT[l.sim]);
-            for (size_t v = 0; v < l.from.size(); ++v) {
-                DevEntR en = P->resE[(size_t)l.e0 + v];
+            P->resAt.push_back(P->resAt[l.sim]);
+            const size_t e0 = (size_t)P->resE0[l.sim], ne = l.from.size();
+            for (size_t v = 0; v < ne; ++v) {
+                DevEntR en = P->resE[e0 + v];
                 en.w = meas[l.from[v]].re;
                 P->resE.push_back(en);
             }
             continue;
         }
-        Like made{si, (int64_t)P->resE.size(), meas, {}};
+        Like made{si, &meas, {}};
+        P->resAt.push_back((int)P->resNT.size());
+        std::fill(rec.begin(), rec.end(), DevResWarp{});
         // the place of an entry: CTA, warp record, lane, row and element of the block
         auto place = [&](const Entry &e, int *cta, int *lane, int *row, int *el) -> DevResWarp & {
             const int i = (int)(e.idx % nx), j = (int)((e.idx / nx - q->shift + ny) % ny);   // the cluster's row
@@ -332,11 +334,7 @@ static void choose_resident(casimir_plan_t *P)
             P->res = q;
             return;
         }
-    P->resW.clear();
-    P->resC.clear();
-    P->resE.clear();
-    P->resT.clear();
-    P->resNT.clear();
+    P->clear_resident();
 }
 
 // allow_resident: the caller left steps_per_launch to the default
@@ -399,7 +397,6 @@ static int prepare_plan(casimir_plan_t *P, bool allow_resident)
     int64_t off = 0;
     std::map<int, std::vector<int>> march_variants;   // per geometry: kernel variant of each march tile
     std::map<int, std::vector<int>> mar2_variants;    // per geometry: variant of each two-step march tile
-    int64_t rese = 0;                                 // entries of the resident march so far
     for (size_t s = 0; s < D.sims.size(); ++s) {
         const Sim &sm = D.sims[s];
         const Geo &g = D.geos[sm.geo];
@@ -443,10 +440,7 @@ static int prepare_plan(casimir_plan_t *P, bool allow_resident)
             for (const Entry &e : sm.src) P->src.push_back(DevSrc{hs.field_off + e.arr * N + e.idx, e.re});
             hs.nsrc = (int)P->src.size() - hs.src0;
             if (P->resident) {
-                hs.resw0 = (int64_t)s * P->res.cluster * (P->res.threads / 32);
-                hs.resc0 = (int64_t)s * P->res.cluster;
-                hs.rese0 = rese;
-                for (int v = 0; v < P->res.cluster; ++v) rese += P->resC[hs.resc0 + v].ne;
+                // its tables are made (resident_tables)
             } else {
                 // multi-step tiles: tile_xk(K) wide for K steps per launch, entries sorted by row with
                 // per-row offsets
@@ -591,10 +585,7 @@ static int prepare_plan(casimir_plan_t *P, bool allow_resident)
                         for (int c = 0; c < 3; ++c)
                             if (g.lorentz[((size_t)id * g.npoles + q) * 6 + 2 * c] != 0.0) geo_poles = std::max(geo_poles, q + 1);
                 if (P->resident) {
-                    hs.resw0 = (int64_t)s * P->res.cluster * (P->res.threads / 32);
-                    hs.resc0 = (int64_t)s * P->res.cluster;
-                    hs.rese0 = rese;
-                    for (int v = 0; v < P->res.cluster; ++v) rese += P->resC[hs.resc0 + v].ne;
+                    // its tables are made (resident_tables)
                 } else if (P->opts.steps_per_launch >= 2 && (hs.cyl || (!P->fp64 && geo_poles <= 1))) {
                     // MARCH_W2-wide strips, entries sorted by row with per-row offsets (the sigma
                     // group is projected from registers)
@@ -1160,16 +1151,17 @@ static int rebuild(casimir_ctx *c)
                                             res[gi].first.cluster == q.cluster && res[gi].first.threads == q.threads && res[gi].first.smem == q.smem)) ++gi;
                 if (gi == res.size()) res.push_back({q, {}});
                 auto ext = [&](DevRes &d) {
-                    d.warps = P->dev.resw + hs.resw0;
-                    d.ctas = P->dev.resc + hs.resc0;
-                    d.ents = P->dev.rese + hs.rese0;
+                    const int64_t at = P->resAt[s];
+                    d.warps = P->dev.resw + at * q.cluster * (q.threads / 32);
+                    d.ctas = P->dev.resc + at * q.cluster;
+                    d.ents = P->dev.rese + P->resE0[s];
                     d.status = r->status_word();
                     d.gen_words = q.gen_words;
                     d.stage_words = q.stage_words;
                     d.ne_max = q.ne_max;
                     d.shift = q.shift;
-                    d.tile_pieces = P->dev.rest + s * (RES_TILES + 1);
-                    d.ntile = P->resNT[s];
+                    d.tile_pieces = P->dev.rest + at * (RES_TILES + 1);
+                    d.ntile = P->resNT[at];
                     d.np_max = q.np_max;
                     d.ntile_max = q.ntile_max;
                     d.term_off = ((q.cyl ? 6 : 3) * (int64_t)hs.nx * hs.ny * (int64_t)P->rsize + 7) / 8;   // the second field buffer

@@ -62,7 +62,6 @@ struct HostSim {
     int tile2_0, ntile2;   // range in the plan's two-step tile list (2D)
     int ent0, nent;        // range in the plan's entry list (bucketed by tile)
     int src0, nsrc;        // range in the plan's source list
-    int64_t resw0 = 0, resc0 = 0, rese0 = 0;   // resident runs: first warp record, CTA record and entry of the simulation
 };
 
 struct HostTile {
@@ -127,11 +126,25 @@ struct casimir_plan {
     int k2d = 1;                      // time steps per launch of the 2D kernel (1, 2 or 3)
     bool resident = false;            // 2D TM/TE plan on the resident march
     Res2dShape res{};
-    std::vector<DevResWarp> resW;     // per simulation, [cluster rank][warp]
-    std::vector<DevResCta> resC;      // per simulation, [cluster rank]
+    // its tables: simulation s has those of number resAt[s], with its own weights from entry resE0[s] on
+    std::vector<int> resAt;
+    std::vector<int64_t> resE0;
     std::vector<DevEntR> resE;
-    std::vector<short> resT;          // per simulation, RES_TILES + 1: first piece of each tile
-    std::vector<int> resNT;           // per simulation: tiles
+    std::vector<DevResWarp> resW;     // per number, [cluster rank][warp]
+    std::vector<DevResCta> resC;      // per number, [cluster rank]
+    std::vector<short> resT;          // per number, RES_TILES + 1: first piece of each tile
+    std::vector<int> resNT;           // per number: tiles
+    void clear_resident()
+    {
+        resident = false;
+        resAt.clear();
+        resE0.clear();
+        resE.clear();
+        resW.clear();
+        resC.clear();
+        resT.clear();
+        resNT.clear();
+    }
     std::vector<HostTile6> tiles6;
     std::vector<HostTile> tilesM;     // march kernel strip tiles (MARCH_W x MARCH_H) with their entries
     std::vector<DevEnt> entsM;

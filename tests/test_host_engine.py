@@ -170,3 +170,14 @@ def test_a_failed_resident_run_stops_at_its_chunk(fake, how):
     fake.fake_fail_resident(0)
     pl.run()                    # the next run's status is its own
     c.close()
+
+
+@pytest.mark.parametrize("make", [lambda: W.piston_small(n_steps=60, precision="fp32"), lambda: W.piston_small(n_steps=60, precision="fp64"),
+                                  lambda: W.cylinder_piston(20, [0, 1, 2], t_max=3.0, n_harm=20, precision="fp64")])
+def test_harmonics_of_a_face_share_their_resident_tables(fake, make):
+    # the tables of a simulation's layout are one per lattice, face and source component, not one per harmonic
+    c = pk.Context(0)
+    resident = c.plan(make()).info()
+    other = c.plan(make(), options={"steps_per_launch": 2}).info()
+    assert resident["device_bytes"] <= 1.005 * other["device_bytes"]
+    c.close()
