@@ -261,12 +261,15 @@ int casimir_plan_site_poles(const casimir_plan_t *plan, int kpoint, int comp, in
 int casimir_plan_pml(const casimir_plan_t *plan, int axis, int half, double *b, double *c,
                      double *inv_kappa);
 
+#define CASIMIR_RESIDENT 1
+
 /* Execution options of a plan (how the leapfrog of Sec. III A is scheduled; the computed
  * force does not depend on them beyond rounding).  0 in a field selects the default. */
 typedef struct {
     int steps_per_launch;   /* time steps fused into one pass over memory: 2D TM/TE runs 1, 2 or 3
                                (default 3 for FP32 runs, 2 for FP64 runs); cylindrical runs 1 or 2
-                               (any value >= 2 fuses two; the default fuses two); other 2D
+                               (any value >= 2 fuses two; the default fuses two), where a resident
+                               march (below) does not take the run; other 2D
                                six-component runs in FP32 whose materials have at most one
                                Lorentz pole 1 or 2 (any value >= 2 fuses two; the default fuses
                                two); all other six-component runs take one step per launch */
@@ -274,7 +277,12 @@ typedef struct {
     int kernel_3d;          /* 3D runs: 3 = column march, both half steps per pass (the default without
                                CPML); 1 = x-line kernel, one half step per pass (the default with
                                CPML); 2 = one-thread-per-cell kernel */
-    int reserved;
+    int reserved;           /* 0, or CASIMIR_RESIDENT (2D TM/TE and cylindrical runs): the march that holds
+                               each simulation's fields on the chip through up to 192 time steps.  The
+                               default takes it where grid and surface fit it, if steps_per_launch is 0
+                               and the environment does not set CASIMIR_STEP2D_K; CASIMIR_RESIDENT: where
+                               they fit it, whatever steps_per_launch says.  casimir_plan_get_options:
+                               CASIMIR_RESIDENT if the plan runs on it */
 } casimir_plan_options;
 
 /* casimir_plan with explicit options (NULL: defaults).  CASIMIR_EINVAL for values out of range. */

@@ -93,7 +93,7 @@ class PlanInfo(ctypes.Structure):
 
 class PlanOptions(ctypes.Structure):
     _fields_ = [("steps_per_launch", ctypes.c_int), ("march_rows", ctypes.c_int), ("kernel_3d", ctypes.c_int),
-                ("reserved", ctypes.c_int)]
+                ("resident", ctypes.c_int)]      # (named reserved in the header)
 
 
 class Stats(ctypes.Structure):
@@ -323,9 +323,11 @@ class Plan:
             ctx._handles.add(h.value)
 
     def options(self):
+        """The options the plan was prepared with, after defaults and autotuning; "resident": 1 among them if the
+        plan runs on a resident march.  Planning with them gives the same plan."""
         o = PlanOptions()
         check(lib().casimir_plan_get_options(self.h, ctypes.byref(o)))
-        return {f: getattr(o, f) for f, _ in PlanOptions._fields_ if f != "reserved"}
+        return {f: getattr(o, f) for f, _ in PlanOptions._fields_ if f != "resident" or o.resident}
 
     def info(self):
         i = PlanInfo()

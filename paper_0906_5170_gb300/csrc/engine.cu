@@ -337,7 +337,7 @@ static void choose_resident(casimir_plan_t *P)
     P->clear_resident();
 }
 
-// allow_resident: the caller left steps_per_launch to the default
+// allow_resident: the caller asked for the resident march, or left steps_per_launch to the default
 static int prepare_plan(casimir_plan_t *P, bool allow_resident)
 {
     PlanData &D = P->data;
@@ -393,6 +393,7 @@ static int prepare_plan(casimir_plan_t *P, bool allow_resident)
         P->pml_off.push_back(po);
     }
     if (allow_resident) choose_resident(P);
+    P->opts.reserved = P->resident ? CASIMIR_RESIDENT : 0;
     // sims, tiles, entries, sources
     int64_t off = 0;
     std::map<int, std::vector<int>> march_variants;   // per geometry: kernel variant of each march tile
@@ -1871,7 +1872,7 @@ static int resolve_options(const casimir_plan_options *in, casimir_plan_options 
     if (o.steps_per_launch < 1 || o.steps_per_launch > 3 || o.march_rows < 1 || o.march_rows > MARCH_H_MAX ||
         o.kernel_3d < 1 || o.kernel_3d > 3)
         return fail(CASIMIR_EINVAL, "plan options out of range");
-    o.reserved = 0;
+    o.reserved = in && in->reserved == CASIMIR_RESIDENT ? CASIMIR_RESIDENT : 0;
     *out = o;
     return CASIMIR_OK;
 }
@@ -1886,7 +1887,7 @@ static int make_plan(casimir_ctx_t *c, const casimir_problem *p, const casimir_p
     if (rc) { delete P; return rc; }
     // a number of time steps per launch, asked for in the options or by the environment, names a
     // kernel of that many; the default leaves 2D TM/TE runs to the resident march where it fits
-    const bool resident = (!opts || opts->steps_per_launch == 0) && !std::getenv("CASIMIR_STEP2D_K");
+    const bool resident = P->opts.reserved == CASIMIR_RESIDENT || ((!opts || opts->steps_per_launch == 0) && !std::getenv("CASIMIR_STEP2D_K"));
     std::string err;
     rc = build_plan(p, &P->data, &err);
     if (rc) { delete P; return fail(rc, err); }

@@ -181,3 +181,31 @@ def test_harmonics_of_a_face_share_their_resident_tables(fake, make):
     other = c.plan(make(), options={"steps_per_launch": 2}).info()
     assert resident["device_bytes"] <= 1.005 * other["device_bytes"]
     c.close()
+
+
+@pytest.mark.parametrize("p,kernel,other", [
+    (W.piston_small(n_steps=60, precision="fp32"), b"k_res2d", b"k_step2d"),
+    (W.piston_small(n_steps=60, precision="fp64"), b"k_res2d", b"k_step2d"),
+    (W.cylinder_piston(10, [0, 1], t_max=2.0), b"k_rescyl", b"k_cyl")])
+def test_options_of_a_plan_give_the_same_plan(fake, p, kernel, other):
+    c = pk.Context(0)
+    o = c.plan(p).options()
+    assert o["resident"] == 1
+    pl = c.plan(p, options=o)
+    assert pl.options() == o
+    fake.fake_reset()
+    pl.run()
+    assert fake.fake_launches(kernel) > 0 and fake.fake_launches(other) == 0
+    # a number of steps per launch alone still names a kernel of that many
+    o.pop("resident")
+    pl = c.plan(p, options=o)
+    assert pl.options() == o
+    fake.fake_reset()
+    pl.run()
+    assert fake.fake_launches(kernel) == 0 and fake.fake_launches(other) > 0
+    # asked for where it does not fit: the kernel of that many steps
+    big = W.config2_piston(W.config2_heights()[0], n_harm=1, n_steps=12)
+    big["n"] = [400, 1000, 1]
+    o = c.plan(big, options={"steps_per_launch": 3, "resident": 1}).options()
+    assert o["steps_per_launch"] == 3 and "resident" not in o
+    c.close()
