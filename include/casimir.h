@@ -293,8 +293,9 @@ int casimir_plan_get_options(const casimir_plan_t *plan, casimir_plan_options *o
 
 /* Autotuning (on != 0): casimir_plan then picks the options itself.  For the first problem of
  * each class (dimension, polarisation family, precision, coordinates, CPML and Lorentz media,
- * complex fields, grid size to a factor of two) it runs every candidate option set on a copy of
- * the problem cut to 128 steps, times the step kernels with CUDA events and keeps the fastest;
+ * complex fields, grid size to a factor of two, whether a resident march takes it) it runs every
+ * candidate option set on a copy of the problem cut to 128 steps, times the step kernels with CUDA
+ * events and keeps the fastest (the default unless another is 3% faster);
  * later problems of the class reuse the choice.  Trials run only while the context is idle
  * (otherwise the defaults apply and nothing is cached).  Off by default. */
 int casimir_ctx_set_autotune(casimir_ctx_t *ctx, int on);

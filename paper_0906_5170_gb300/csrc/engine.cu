@@ -337,12 +337,9 @@ static void choose_resident(casimir_plan_t *P)
     P->clear_resident();
 }
 
-// allow_resident: the caller asked for the resident march, or left steps_per_launch to the default
-static int prepare_plan(casimir_plan_t *P, bool allow_resident)
+static int prepare_plan(casimir_plan_t *P)
 {
     PlanData &D = P->data;
-    P->fp64 = D.prob.precision == CASIMIR_FP64;
-    P->rsize = P->fp64 ? 8 : 4;
     // geometry tables
     for (auto &g : D.geos) {
         P->mat_off.push_back((int64_t)P->mat_all.size());
@@ -392,8 +389,6 @@ static int prepare_plan(casimir_plan_t *P, bool allow_resident)
             }
         P->pml_off.push_back(po);
     }
-    if (allow_resident) choose_resident(P);
-    P->opts.reserved = P->resident ? CASIMIR_RESIDENT : 0;
     // sims, tiles, entries, sources
     int64_t off = 0;
     std::map<int, std::vector<int>> march_variants;   // per geometry: kernel variant of each march tile
@@ -1877,28 +1872,45 @@ static int resolve_options(const casimir_plan_options *in, casimir_plan_options 
     return CASIMIR_OK;
 }
 
+using PlanPtr = std::unique_ptr<casimir_plan_t>;
+
+// A plan up to the choice of its kernel.  A number of time steps per launch, asked for in the options or by the
+// environment, names a kernel of that many; the default leaves 2D TM/TE and cylindrical runs to the resident march
+// where it fits.
+static int begin_plan(casimir_ctx_t *c, const casimir_problem *p, const casimir_plan_options *opts, PlanPtr *out)
+{
+    PlanPtr P(new casimir_plan_t());
+    P->ctx = c;
+    int rc = resolve_options(opts, &P->opts, p->precision == CASIMIR_FP64, has_pml3d(*p));
+    if (rc) return rc;
+    std::string err;
+    rc = build_plan(p, &P->data, &err);
+    if (rc) return fail(rc, err);
+    P->fp64 = P->data.prob.precision == CASIMIR_FP64;
+    P->rsize = P->fp64 ? 8 : 4;
+    if (P->opts.reserved == CASIMIR_RESIDENT || ((!opts || opts->steps_per_launch == 0) && !std::getenv("CASIMIR_STEP2D_K"))) choose_resident(P.get());
+    *out = std::move(P);
+    return CASIMIR_OK;
+}
+
+static int end_plan(PlanPtr P, casimir_plan_t **out)
+{
+    P->opts.reserved = P->resident ? CASIMIR_RESIDENT : 0;
+    int rc = prepare_plan(P.get());
+    if (rc) return rc;
+    if (P->ctx && (uint64_t)(P->table_bytes + P->request_bytes) > P->ctx->budget)
+        return fail(CASIMIR_ENOMEM, "plan needs more device memory than the context budget");
+    *out = P.release();
+    return CASIMIR_OK;
+}
+
 static int make_plan(casimir_ctx_t *c, const casimir_problem *p, const casimir_plan_options *opts, casimir_plan_t **out)
 {
     NvtxRange nvtx_("casimir.plan");
     *out = nullptr;
-    auto *P = new casimir_plan_t();
-    P->ctx = c;
-    int rc = resolve_options(opts, &P->opts, p->precision == CASIMIR_FP64, has_pml3d(*p));
-    if (rc) { delete P; return rc; }
-    // a number of time steps per launch, asked for in the options or by the environment, names a
-    // kernel of that many; the default leaves 2D TM/TE runs to the resident march where it fits
-    const bool resident = P->opts.reserved == CASIMIR_RESIDENT || ((!opts || opts->steps_per_launch == 0) && !std::getenv("CASIMIR_STEP2D_K"));
-    std::string err;
-    rc = build_plan(p, &P->data, &err);
-    if (rc) { delete P; return fail(rc, err); }
-    rc = prepare_plan(P, resident);
-    if (rc) { delete P; return rc; }
-    if (c && (uint64_t)(P->table_bytes + P->request_bytes) > c->budget) {
-        delete P;
-        return fail(CASIMIR_ENOMEM, "plan needs more device memory than the context budget");
-    }
-    *out = P;
-    return CASIMIR_OK;
+    PlanPtr P;
+    const int rc = begin_plan(c, p, opts, &P);
+    return rc ? rc : end_plan(std::move(P), out);
 }
 
 // Problem class for autotuning: what decides which schedule is fastest.
@@ -1916,16 +1928,17 @@ static std::string tune_key(const casimir_problem &p)
     return k;
 }
 
-// Time each candidate on the problem cut to 128 steps; the fastest per cell-update wins.
-static casimir_plan_options autotune(casimir_ctx *c, const casimir_problem &p)
+// Time each candidate on the problem cut to 128 steps; the fastest per cell-update wins, or the default (the first:
+// all options 0) unless it is 3% slower.  resident: the default plan runs on a resident march; such problems are
+// classes of their own, since a choice made for a grid too large for a cluster says nothing about them.
+static casimir_plan_options autotune(casimir_ctx *c, const casimir_problem &p, bool resident)
 {
     NvtxRange nvtx_("casimir.autotune");
     casimir_plan_options dflt{};
     resolve_options(nullptr, &dflt, p.precision == CASIMIR_FP64, has_pml3d(p));
-    std::vector<casimir_plan_options> cand;
+    std::vector<casimir_plan_options> cand = {casimir_plan_options{}};
     if (p.dims == 3) {
-        // the default first (ties keep it), then the other 3D kernels
-        cand = {dflt};
+        // the other 3D kernels
         for (int k : {3, 1, 2})
             if (k != dflt.kernel_3d) {
                 casimir_plan_options o = dflt;
@@ -1934,6 +1947,7 @@ static casimir_plan_options autotune(casimir_ctx *c, const casimir_problem &p)
             }
     } else if (p.polarization == CASIMIR_POL_FULL) {
         for (int rows : {32, 16, 64}) {
+            if (!resident && rows == dflt.march_rows) continue;   // the default
             casimir_plan_options o = dflt;
             o.march_rows = rows;
             cand.push_back(o);
@@ -1946,16 +1960,15 @@ static casimir_plan_options autotune(casimir_ctx *c, const casimir_problem &p)
             cand.push_back(o);
         }
     } else {
-        // the default first (ties keep it: the resident march where it fits), then the fusion depths
-        cand = {casimir_plan_options{}, dflt};
+        // the fusion depths
         for (int k : {3, 2, 1})
-            if (k != dflt.steps_per_launch) {
+            if (resident || k != dflt.steps_per_launch) {
                 casimir_plan_options o = dflt;
                 o.steps_per_launch = k;
                 cand.push_back(o);
             }
     }
-    const std::string key = tune_key(p);
+    const std::string key = tune_key(p) + (resident ? "r" : "");
     {
         std::lock_guard<std::mutex> lk(c->mu);
         auto it = c->tuned.find(key);
@@ -1967,7 +1980,7 @@ static casimir_plan_options autotune(casimir_ctx *c, const casimir_problem &p)
     // the context's statistics belong to its user: restore them after the trials
     const double ms0 = c->step_ms;
     const int64_t l0 = c->step_launches, cu0 = c->cell_updates;
-    double best_t = 0;
+    double best_t = 0, dflt_t = 0;
     casimir_plan_options best{};
     bool any = false;
     for (const casimir_plan_options &o : cand) {
@@ -1982,8 +1995,10 @@ static casimir_plan_options autotune(casimir_ctx *c, const casimir_problem &p)
         casimir_plan_destroy(tp);
         if (rc != CASIMIR_OK || dcu <= 0) continue;
         const double t = dms / (double)dcu;
+        if (&o == &cand[0]) dflt_t = t;
         if (!any || t < best_t) { best_t = t; best = o; any = true; }
     }
+    if (dflt_t > 0 && best_t > 0.97 * dflt_t) best = casimir_plan_options{};
     c->step_ms = ms0;
     c->step_launches = l0;
     c->cell_updates = cu0;
@@ -2012,7 +2027,16 @@ int casimir_plan(casimir_ctx_t *c, const casimir_problem *p, casimir_plan_t **ou
     // nothing thrown by the planner (host allocation, thread creation) crosses the C ABI
     try {
         if (c && c->autotune) {
-            const casimir_plan_options o = autotune(c, *p);
+            *out = nullptr;
+            PlanPtr P;
+            if (p->dims == 2 && (p->polarization != CASIMIR_POL_FULL || p->coords == CASIMIR_COORDS_CYLINDRICAL)) {
+                // the class depends on whether the resident march takes the default plan
+                const int rc = begin_plan(c, p, nullptr, &P);
+                if (rc) return rc;
+            }
+            const casimir_plan_options o = autotune(c, *p, P && P->resident);
+            if (P && o.steps_per_launch == 0) return end_plan(std::move(P), out);
+            P.reset();
             return make_plan(c, p, &o, out);
         }
         return make_plan(c, p, nullptr, out);

@@ -209,3 +209,47 @@ def test_options_of_a_plan_give_the_same_plan(fake, p, kernel, other):
     o = c.plan(big, options={"steps_per_launch": 3, "resident": 1}).options()
     assert o["steps_per_launch"] == 3 and "resident" not in o
     c.close()
+
+
+def _cell(nx, ny, steps=200):
+    p = W._base(2, (nx, ny, 1), 10.0, steps)
+    p["faces"] = W.box_faces([3.0, 3.0], [6.0, 5.0], 2)
+    p.update(n_harm=1, polarization="TE+TM", precision="fp32", force_axis=0)
+    return p
+
+
+def test_autotuning_knows_the_resident_marches(fake):
+    c = pk.Context(0)
+    c.set_autotune(True)
+    cyl = W.cylinder_piston(10, [0, 1], t_max=2.0)
+    # a class keeps the default unless another candidate is clearly faster
+    fake.fake_cost(b"k_rescyl", 64 * 0.010)
+    fake.fake_cost(b"k_march6", 0.0099)
+    fake.fake_cost(b"k_cyl2", 0.0099)
+    pl = c.plan(cyl)
+    assert pl.options()["resident"] == 1
+    fake.fake_reset()
+    pl.run()
+    assert fake.fake_launches(b"k_rescyl") > 0
+    assert c.plan(W.cylinder_piston(10, [0, 1], t_max=2.0, below=0.4)).options()["resident"] == 1
+    # a grid too large for a cluster and a smaller one of the same class (size to a factor of two)
+    fake.fake_reset()
+    fake.fake_cost(b"k_step2d_tk", 0.0101)
+    fake.fake_cost(b"k_step2d", 0.010)
+    assert "resident" not in c.plan(_cell(400, 500)).options()
+    # each kernel tried once: 43 launches of three steps, 64 of two, 128 of one
+    assert fake.fake_launches(b"k_step2d_tk") == 43
+    pl = c.plan(_cell(400, 280))
+    assert pl.options()["resident"] == 1
+    c.close()
+    # clearly faster: it is kept, for both
+    c = pk.Context(0)
+    c.set_autotune(True)
+    fake.fake_reset()
+    fake.fake_cost(b"k_rescyl", 64 * 0.010)
+    fake.fake_cost(b"k_march6", 0.010)
+    fake.fake_cost(b"k_cyl2", 0.002)
+    for below in (0.5, 0.4):
+        o = c.plan(W.cylinder_piston(10, [0, 1], t_max=2.0, below=below)).options()
+        assert "resident" not in o and o["steps_per_launch"] in (1, 2)
+    c.close()
