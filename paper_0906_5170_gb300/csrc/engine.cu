@@ -1876,8 +1876,8 @@ using PlanPtr = std::unique_ptr<casimir_plan_t>;
 
 // A plan up to the choice of its kernel.  A number of time steps per launch, asked for in the options or by the
 // environment, names a kernel of that many; the default leaves 2D TM/TE and cylindrical runs to the resident march
-// where it fits.
-static int begin_plan(casimir_ctx_t *c, const casimir_problem *p, const casimir_plan_options *opts, PlanPtr *out)
+// where it fits (resident false: to the multi-step kernels).
+static int begin_plan(casimir_ctx_t *c, const casimir_problem *p, const casimir_plan_options *opts, bool resident, PlanPtr *out)
 {
     PlanPtr P(new casimir_plan_t());
     P->ctx = c;
@@ -1888,18 +1888,25 @@ static int begin_plan(casimir_ctx_t *c, const casimir_problem *p, const casimir_
     if (rc) return fail(rc, err);
     P->fp64 = P->data.prob.precision == CASIMIR_FP64;
     P->rsize = P->fp64 ? 8 : 4;
-    if (P->opts.reserved == CASIMIR_RESIDENT || ((!opts || opts->steps_per_launch == 0) && !std::getenv("CASIMIR_STEP2D_K"))) choose_resident(P.get());
+    if (resident && (P->opts.reserved == CASIMIR_RESIDENT || ((!opts || opts->steps_per_launch == 0) && !std::getenv("CASIMIR_STEP2D_K")))) choose_resident(P.get());
     *out = std::move(P);
     return CASIMIR_OK;
 }
 
-static int end_plan(PlanPtr P, casimir_plan_t **out)
+// Its tables; a resident plan whose tables do not fit the budget becomes one of the multi-step kernels, whose
+// tables can be a little smaller.
+static int end_plan(PlanPtr P, const casimir_problem *p, const casimir_plan_options *opts, casimir_plan_t **out)
 {
     P->opts.reserved = P->resident ? CASIMIR_RESIDENT : 0;
+    casimir_ctx *c = P->ctx;
     int rc = prepare_plan(P.get());
     if (rc) return rc;
-    if (P->ctx && (uint64_t)(P->table_bytes + P->request_bytes) > P->ctx->budget)
-        return fail(CASIMIR_ENOMEM, "plan needs more device memory than the context budget");
+    if (c && (uint64_t)(P->table_bytes + P->request_bytes) > c->budget) {
+        if (!P->resident) return fail(CASIMIR_ENOMEM, "plan needs more device memory than the context budget");
+        P.reset();
+        rc = begin_plan(c, p, opts, false, &P);
+        return rc ? rc : end_plan(std::move(P), p, opts, out);
+    }
     *out = P.release();
     return CASIMIR_OK;
 }
@@ -1909,8 +1916,8 @@ static int make_plan(casimir_ctx_t *c, const casimir_problem *p, const casimir_p
     NvtxRange nvtx_("casimir.plan");
     *out = nullptr;
     PlanPtr P;
-    const int rc = begin_plan(c, p, opts, &P);
-    return rc ? rc : end_plan(std::move(P), out);
+    const int rc = begin_plan(c, p, opts, true, &P);
+    return rc ? rc : end_plan(std::move(P), p, opts, out);
 }
 
 // Problem class for autotuning: what decides which schedule is fastest.
@@ -2031,11 +2038,11 @@ int casimir_plan(casimir_ctx_t *c, const casimir_problem *p, casimir_plan_t **ou
             PlanPtr P;
             if (p->dims == 2 && (p->polarization != CASIMIR_POL_FULL || p->coords == CASIMIR_COORDS_CYLINDRICAL)) {
                 // the class depends on whether the resident march takes the default plan
-                const int rc = begin_plan(c, p, nullptr, &P);
+                const int rc = begin_plan(c, p, nullptr, true, &P);
                 if (rc) return rc;
             }
             const casimir_plan_options o = autotune(c, *p, P && P->resident);
-            if (P && o.steps_per_launch == 0) return end_plan(std::move(P), out);
+            if (P && o.steps_per_launch == 0) return end_plan(std::move(P), p, nullptr, out);
             P.reset();
             return make_plan(c, p, &o, out);
         }

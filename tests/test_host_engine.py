@@ -253,3 +253,24 @@ def test_autotuning_knows_the_resident_marches(fake):
         o = c.plan(W.cylinder_piston(10, [0, 1], t_max=2.0, below=below)).options()
         assert "resident" not in o and o["steps_per_launch"] in (1, 2)
     c.close()
+
+
+def test_a_budget_that_held_the_multi_step_plan_still_does(fake):
+    p = W.piston_small(n_steps=60, precision="fp64")
+    c = pk.Context(0)
+    resident, other = c.plan(p).info()["device_bytes"], c.plan(p, options={"steps_per_launch": 2}).info()["device_bytes"]
+    c.close()
+    assert resident > other
+    for autotune in (False, True):
+        c = pk.Context(0, hbm_budget_bytes=other)
+        c.set_autotune(autotune)
+        pl = c.plan(p)
+        assert "resident" not in pl.options()
+        pl.run()
+        pl.close()
+        c.close()
+    c = pk.Context(0, hbm_budget_bytes=other - 1)
+    with pytest.raises(pk.CasimirError) as e:
+        c.plan(p)
+    assert e.value.code == pk.capi.ENOMEM
+    c.close()
