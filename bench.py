@@ -30,14 +30,16 @@ sys.path.insert(0, ROOT)
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per cell of one launch, from one ncu capture of
 # the kernel on the piston profiling case (`--profile-case piston`, 17.0 M cells, above L2).  Traffic grows in
 # proportion to the cells (same tiles, same access pattern), so the benchmark's launch scales by its cell count.
-# Each entry records the kernel source it was captured from and that file's SHA-256 prefix at capture time:
-# when the source has changed since, the bench reports the traffic as null (stale) instead of a wrong figure.
+# Each entry records the kernel sources it was captured from and the SHA-256 prefix of their concatenation at
+# capture time: when a source has changed since, the bench reports the traffic as null (stale) instead of a wrong
+# figure.
 DRAM_BYTES_PER_CELL_LAUNCH = {
     "k_step2d_tk<float, 3>": {"bytes_per_cell": (211.063e6 + 162.221e6) / 16998400,
-                              "source": "paper_0906_5170_gb300/csrc/step2d_tk.cu", "sha256_16": "78d8356d7697ee99",
+                              "sources": ["paper_0906_5170_gb300/csrc/step2d_tk.cu"], "sha256_16": "78d8356d7697ee99",
                               "profile": "profiles/k_step2d_tk_piston_sweep.md"},
-    "k_res2d<float>": {"bytes_per_cell": (206.963e6 + 150.095e6) / 16998400,
-                       "source": "paper_0906_5170_gb300/csrc/res2d.cu", "sha256_16": "efcf87a30f636a43",
+    "k_res2d<float>": {"bytes_per_cell": (204.764e6 + 149.049e6) / 16998400,
+                       "sources": ["paper_0906_5170_gb300/csrc/res2d.cu", "paper_0906_5170_gb300/csrc/resident.cuh"],
+                       "sha256_16": "6476ec3f4abe4c8c",
                        "profile": "profiles/k_res2d_piston_sweep.md"},
 }
 
@@ -49,11 +51,53 @@ def traffic_per_cell(kernel):
     e = DRAM_BYTES_PER_CELL_LAUNCH.get(kernel)
     if not e:
         return None, None
-    with open(os.path.join(ROOT, e["source"]), "rb") as f:
-        h = hashlib.sha256(f.read()).hexdigest()[:16]
-    prov = {"profile": e["profile"], "source": e["source"], "source_sha256_16": h, "captured_sha256_16": e["sha256_16"],
+    h = hashlib.sha256()
+    for src in e["sources"]:
+        with open(os.path.join(ROOT, src), "rb") as f:
+            h.update(f.read())
+    h = h.hexdigest()[:16]
+    prov = {"profile": e["profile"], "sources": e["sources"], "source_sha256_16": h, "captured_sha256_16": e["sha256_16"],
             "stale": h != e["sha256_16"]}
     return (None if prov["stale"] else e["bytes_per_cell"]), prov
+
+
+RES_LAUNCH_INDICES = 64      # launch indices of one resident launch at most (csrc/kernels.h)
+
+
+def roofline(plans, steps, launches, step_ms, cell_updates, bytes_per_update, hbm, peak_kind):
+    """The step kernel of the timed region against the measured copy bandwidth.  plans: (options, info) of each plan of a
+    step; launches, step_ms, cell_updates: the context's kernel statistics over `steps` steps.
+
+    Multi-step kernels launch once per launch index for all plans together.  Resident marches launch once per chunk
+    of up to 64 indices and per shape (`groups`), the shapes of a chunk side by side: they count as one launch here."""
+    resident = all(o.get("resident") for o, _ in plans)
+    kmax = max(o["steps_per_launch"] for o, _ in plans)
+    if resident:
+        kernel, of = "k_res2d<float>", "up to 192 time steps"
+        cells = sum(i["n_cells"] for _, i in plans)
+        each = steps * max(-(-i["launches"] // RES_LAUNCH_INDICES) for _, i in plans)   # of one shape, at least
+        groups = max(1, min(launches // each, len(plans)))
+    else:
+        kernel = {1: "k_step2d<float>", 2: "k_step2d_t2<float>", 3: "k_step2d_tk<float, 3>"}[kmax]
+        of = f"{kmax} time step{'s' if kmax > 1 else ''}"
+        cells = sum(i["n_cells"] for o, i in plans if o["steps_per_launch"] == kmax)
+        groups = 1
+    per_cell, prov = traffic_per_cell(kernel)
+    achieved = cell_updates * bytes_per_update / (step_ms / 1e3) / 1e9 if step_ms > 0 else None
+    launch_ms = step_ms / max(1, launches / groups)
+    # what bounds the kernel: memory, or (fields in registers through a launch) the latency of a step's chain;
+    # achieved and frac are algorithmic bytes against the copy bandwidth in both cases.  Several time steps per pass over
+    # memory lift them above the copy peak; the DRAM traffic ncu measured for the kernel shows what HBM really moves.
+    roof = {"bound": "latency" if resident else "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
+            "frac": achieved / hbm if achieved else None,
+            "traffic": per_cell * cells if per_cell else None,
+            "traffic_unit": "bytes per launch (ncu dram read + write per cell, scaled to this launch's cells)",
+            "traffic_provenance": prov, "kernel": f"{kernel} ({of} per launch)", "bytes_per_cell_update": bytes_per_update,
+            "cells_per_launch": cells, "shapes_per_launch": groups, "avg_launch_ms": launch_ms, "peak_source": peak_kind}
+    if per_cell and launches and step_ms > 0:
+        roof["dram_gbs"] = per_cell * cells / (launch_ms / 1e3) / 1e9
+        roof["dram_frac"] = roof["dram_gbs"] / hbm
+    return roof
 
 
 METRIC = "forces/s and Gcell-updates/s (% HBM roofline), p50/p99 latency vs plain at 1e-4 rel"
@@ -708,32 +752,8 @@ def main():
     forces_per_s = n_forces * args.steps * world / (ms / 1e3)
 
     hbm, peak_kind = peaks()
-    b_alg = infos[0]["bytes_per_update"]
-    achieved = cups_kernel * b_alg / (step_ms / 1e3) / 1e9 if step_ms > 0 else None
-    # the step kernel the timed plans ran (their execution options, autotuned or default)
-    kmax = max(pl.options()["steps_per_launch"] for pl in plans)
-    kernel = {1: "k_step2d<float>", 2: "k_step2d_t2<float>", 3: "k_step2d_tk<float, 3>"}[kmax]
-    cells_per_launch = sum(i["n_cells"] for i, pl in zip(infos, plans) if pl.options()["steps_per_launch"] == kmax)
-    # runs left to the default options take the resident march where it fits: one launch per chunk of steps
-    # (fields in registers, DRAM traffic only between launches) instead of one per launch index
-    resident = launches < args.steps * max(i["launches"] for i in infos)
-    if resident:
-        kernel = "k_res2d<float>"
-    per_cell, traffic_prov = traffic_per_cell(kernel)
-    roof = {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
-            "frac": achieved / hbm if achieved else None,
-            "traffic": per_cell * cells_per_launch if per_cell else None,
-            "traffic_unit": "bytes per launch (ncu dram read + write per cell, scaled to this launch's cells)",
-            "traffic_provenance": traffic_prov,
-            "kernel": kernel + (" (up to 192 time steps per launch)" if resident else f" ({kmax} time step{'s' if kmax > 1 else ''} per launch)"),
-            "bytes_per_cell_update": b_alg,
-            "cells_per_launch": cells_per_launch,
-            "avg_launch_ms": step_ms / max(1, launches), "peak_source": peak_kind}
-    # temporal blocking (several time steps per pass over memory) lifts the algorithmic-byte figure
-    # above the copy peak; the DRAM traffic ncu measured for the kernel shows what HBM really moves
-    if per_cell and launches and step_ms > 0:
-        roof["dram_gbs"] = per_cell * cells_per_launch / (step_ms / launches / 1e3) / 1e9
-        roof["dram_frac"] = roof["dram_gbs"] / hbm
+    roof = roofline([(pl.options(), i) for pl, i in zip(plans, infos)], args.steps, launches, step_ms, cups_kernel,
+                    infos[0]["bytes_per_update"], hbm, peak_kind)
 
     e2e = None
     if not args.no_e2e:
