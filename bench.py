@@ -37,9 +37,9 @@ DRAM_BYTES_PER_CELL_LAUNCH = {
     "k_step2d_tk<float, 3>": {"bytes_per_cell": (211.063e6 + 162.221e6) / 16998400,
                               "sources": ["paper_0906_5170_gb300/csrc/step2d_tk.cu"], "sha256_16": "78d8356d7697ee99",
                               "profile": "profiles/k_step2d_tk_piston_sweep.md"},
-    "k_res2d<float>": {"bytes_per_cell": (204.764e6 + 149.049e6) / 16998400,
+    "k_res2d<float>": {"bytes_per_cell": (205.058e6 + 149.596e6) / 16998400,
                        "sources": ["paper_0906_5170_gb300/csrc/res2d.cu", "paper_0906_5170_gb300/csrc/resident.cuh"],
-                       "sha256_16": "6476ec3f4abe4c8c",
+                       "sha256_16": "e6f74717cc0d0d1e",
                        "profile": "profiles/k_res2d_piston_sweep.md"},
 }
 

@@ -204,17 +204,15 @@ k_rescyl(const DevResCyl *__restrict__ sims, int64_t launch, int count)
     auto wait_far = [&](unsigned need, unsigned lead, unsigned mb, int i) {
         if (flags & need) {
             const unsigned m = mb + 8u * (i & 1);
-            if (!(flags & F_DEAD) && !mb_wait(m, ((unsigned)i >> 1) & 1u)) flags |= F_DEAD;
-            // (its phase over: another arrival on an unfinished one would be undefined)
-            if ((flags & (lead | F_DEAD)) == lead && i + 2 < cnt) mb_expect(m, 2 * D.tcols * 16);
+            if (!mb_wait(m, ((unsigned)i >> 1) & 1u)) flags = (flags | F_DEAD) & ~F_EXCHANGE;
+            if ((flags & lead) && i + 2 < cnt) mb_expect(m, 2 * D.tcols * 16);
         }
     };
     auto consume = [&](int i) {
         sums.consume(i, flags & F_MINE, reinterpret_cast<const R *>(blocks + stage_w + (i & 1) * sbuf), (int)(pk_stage >> 16));
     };
-    // (after a wait that ran out nothing is sent: no neighbour may count more bytes than it waits for)
     auto put_row = [&](unsigned far, int at, unsigned cta, unsigned mb, const V4 &v) {
-        if ((flags & (far | F_DEAD)) == far) st_async(map_rank((unsigned)__cvta_generic_to_shared(blocks + at), cta), map_rank(mb, cta), v);
+        if (flags & far) st_async(map_rank((unsigned)__cvta_generic_to_shared(blocks + at), cta), map_rank(mb, cta), v);
         else blocks[at] = v;
     };
     auto col_of = [&](const R (&f)[RB][CX], int c, int k) -> V4 {

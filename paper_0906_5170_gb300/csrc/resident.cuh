@@ -102,6 +102,10 @@ __device__ __noinline__ void linger()
 constexpr unsigned F_ACTIVE = 1u, F_SHORT = 2u, F_FARU = 4u, F_FARD = 8u, F_NEEDU = 16u, F_NEEDD = 32u, F_LEADU = 64u, F_LEADD = 128u,
                    F_LATE = 256u, F_STAGE = 512u, F_MINE = 1024u, F_DEAD = 2048u, F_FIRST = 4096u, F_STAGEW = 8192u;
 constexpr unsigned F_PLAIN = 1u << 23;
+// What a thread whose wait ran out (F_DEAD) takes no further part in: it waits no more, arms no mbarrier (another
+// arrival on an unfinished phase would be undefined) and sends no row (no neighbour may count more bytes than it
+// waits for); its rows go to its own CTA's slots, where nothing reads a failed run's values.
+constexpr unsigned F_EXCHANGE = F_FARU | F_FARD | F_NEEDU | F_NEEDD | F_LEADU | F_LEADD;
 constexpr int RES_WIN = 16;              // steps of a window of the projection
 constexpr int F_W = 14;                  // valid columns less one (2 bits)
 constexpr int F_ROWS = 16;               // staged rows of the block (7 bits)
