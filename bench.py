@@ -6,7 +6,7 @@ between PEC sidewalls at 8 sidewall separations h in [0.5, 3], grids 400 x
 40(1+2h) at resolution 40, TE + TM, a rectangular stress contour with 40 cosine
 harmonics per face, 20000 time steps, FP32 fields with FP64 accumulation; 8
 forces, 5120 source simulations (640 runs of 8 exactly-pruned simulations), all
-admitted together into one batched launch per time step.
+admitted together into one batch: a launch per grid for every chunk of time steps.
 
 Prints one JSON line.  `--impl reference` times the FP64 CPU oracle instead, on
 a bounded sample of the same workload.
